@@ -748,10 +748,17 @@ fmlbm_status fmlbm_step(fmlbm_handle* h, int64_t nsteps) {
     // may not wait on work outside the capture): a request is then served entirely on the
     // captured stream.
     bool capturing = false;
-    if (nsteps > 0 && h->pending >= 0) {
+    // Each step is launched programmatically behind the one before it (pdl_wait), except under
+    // capture (a graph's launches follow each other without the gaps) and where the step also
+    // waits for the diagnostics stream.
+    bool pdl = false;
+    if (nsteps > 0) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        FM_CUDA(h, cudaStreamIsCapturing(h->stream, &cap));
+        const cudaError_t e = cudaStreamIsCapturing(h->stream, &cap);
+        if (e != cudaSuccess && h->pending >= 0) FM_CUDA(h, e);
+        if (e != cudaSuccess) cudaGetLastError();
         capturing = cap != cudaStreamCaptureStatusNone;
+        pdl = e == cudaSuccess && !capturing;
     }
     for (int64_t k = 0; k < nsteps; ++k) {
         if (nsteps - k >= 2 && h->pending < 0 && resolved_variant(h) == FMLBM_VARIANT_MULTI) {
@@ -775,6 +782,7 @@ fmlbm_status fmlbm_step(fmlbm_handle* h, int64_t nsteps) {
         }
         StepArgs A = make_args(h, h->cur);
         const int64_t fused = h->pending;
+        A.pdl = pdl && fused < 0;
         if (fused >= 0) {  // this step also reduces the state it reads
             A.diag_partial = partial_set(h, fused);
             A.rho_prev = h->rho_prev;

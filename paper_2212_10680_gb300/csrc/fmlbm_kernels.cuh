@@ -141,7 +141,7 @@ struct StepArgs {
     // rows [check_y0, check_y1) whose nodes the domain check covers (check_y1 = 0: all); a slab
     // of a decomposed lattice leaves out its ghost rows, whose update is discarded
     int check_y0, check_y1;
-    int pad0;
+    int pdl;               // host: launch programmatically behind the stream's preceding launch
     long long wait_polls;  // polls of a bounded wait for a tile copy (bulk-copy step forms)
 };
 __device__ __forceinline__ bool checked_row(const StepArgs& A, int y) {
@@ -282,6 +282,17 @@ __device__ __forceinline__ void store_gsel(const StepArgs& A, const Planes* P, i
     if constexpr (PP) store_gp<ST>(*P, i, a, node, v);
     else store_g<ST>(A, i, a, (size_t)node, (size_t)nxy, v);
 }
+
+// Programmatic launch of consecutive steps: a step launched with the stream-serialization
+// attribute is set up while the launch before it drains; pdl_wait, before the first access to
+// memory, blocks until that launch has completed and its stores are visible (at once for an
+// ordinary launch).  Back to back, ordinary launches of a kernel of t us came 2-3 us apart beyond
+// t and only at multiples of 2.05 us on GB300 (t = 3.0: 6.15 us per launch; t = 8.0: 10.25);
+// programmatic ones 0.4 us beyond t.  The steps do not trigger the next launch early
+// (griddepcontrol.launch_dependents): its blocks then took slots from the running step's last
+// wave (20 steps of the 1024^2 binary: 776 us, with a trigger at the start 838 us, 828 us with
+// ordinary launches).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ int wrap(int v, int n) {
     int r = v % n;
@@ -705,8 +716,7 @@ __device__ __forceinline__ void phase2(const MixConstT<Real>& m, StepSmem<Real, 
 
 // Phase 3 at one lane of nodes: force (step 7), velocity (step 1), equilibrium and
 // forcing (step 8) and collision (step 9).
-//   Gt, Rt: the Phi tile (tile + 1) and the rho~ tile (tile + 2); (cx, cy) the node's
-//           position in the tile + 1 coordinates, lane k at cx + k ds;
+//   grads(i, px, py, rx, ry, rti): the gradients of Phi_i and of rho~_i at the node, and rho~_i;
 //   rho, jx, jy: the component densities and the total first moment of step 1 (phase 1);
 //   geth(i, h): the nine pulled values of component i;
 //   Fpx, Fpy: the stored total force F(t - 1) (LAG: the lagged reading; ignored otherwise);
@@ -717,17 +727,13 @@ __device__ __forceinline__ void phase2(const MixConstT<Real>& m, StepSmem<Real, 
 // STD: the standard formulation of Section VI -- equilibrium rho_i w_a [1 + ...] of
 // Eq. eqLBE, Guo's forcing term of Eq. eqLBEfinal3 (no grad rho_i part) and
 // F_i + c_s^2 grad rho_i of Eq. eqForceGen.
-template <int NC, bool COLLIDE, bool STD, bool LAG, typename V, typename E, typename TG, typename TR, typename GetH,
-          typename Store>
-__device__ __forceinline__ void phase3_core(const MixConstT<E>& m, int stencil, const TG& Gt, const TR& Rt, int cx,
-                                            int cy, int ds, const V (&rho)[NC], V jx, V jy, GetH&& geth, V Fpx,
-                                            V Fpy, Store&& store, V& Ftx, V& Fty, V& ux, V& uy) {
+template <int NC, bool COLLIDE, bool STD, bool LAG, typename V, typename E, typename Grads, typename GetH, typename Store>
+__device__ __forceinline__ void phase3_core(const MixConstT<E>& m, Grads&& grads, const V (&rho)[NC], V jx, V jy,
+                                            GetH&& geth, V Fpx, V Fpy, Store&& store, V& Ftx, V& Fty, V& ux, V& uy) {
     // F_i and grad rho_i of component i
     auto force = [&](int i, V& Fx, V& Fy, V& grx, V& gry) {
-        V px, py, rx, ry;
-        grad_at<V>(Gt, i, cx, cy, ds, stencil, px, py);
-        grad_at<V>(Rt, i, cx + 1, cy + 1, ds, stencil, rx, ry);
-        const V rti = tld<V>(Rt, i, cy + 1, cx + 1, ds);
+        V px, py, rx, ry, rti;
+        grads(i, px, py, rx, ry, rti);
         // grad rho_i = M_i grad rho~_i
         grx = vmul(rx, vbc<V>(m.M[i]));
         gry = vmul(ry, vbc<V>(m.M[i]));
@@ -829,6 +835,16 @@ __device__ __forceinline__ void phase3_core(const MixConstT<E>& m, int stencil, 
     }
 }
 
+// The gradients phase 3 needs, from a Phi tile (tile + 1) and a rho~ tile (tile + 2); (cx, cy)
+// the node's position in the tile + 1 coordinates, lane k at cx + k ds.
+template <typename V, typename TG, typename TR>
+__device__ __forceinline__ void tile_grads(const TG& Gt, const TR& Rt, int i, int cx, int cy, int ds, int stencil, V& px,
+                                           V& py, V& rx, V& ry, V& rti) {
+    grad_at<V>(Gt, i, cx, cy, ds, stencil, px, py);
+    grad_at<V>(Rt, i, cx + 1, cy + 1, ds, stencil, rx, ry);
+    rti = tld<V>(Rt, i, cy + 1, cx + 1, ds);
+}
+
 // Phase 3 of the one-node-per-thread kernels at one valid node.
 template <int NC, int ST, int TY, bool MOMENTS, bool STD = false, bool PARK = false, bool PP = false>
 __device__ __forceinline__ void phase3(const StepArgs& A, const MixConstT<typename StoreTraits<ST>::Real>& m,
@@ -846,14 +862,16 @@ __device__ __forceinline__ void phase3(const StepArgs& A, const MixConstT<typena
     auto store = [&](int i, int a, Real v) { store_gsel<ST, PP>(A, P, i, a, node, nxy, v); };
     Real Ftx, Fty, ux, uy;
     const int sten = stencil >= 0 ? stencil : A.stencil;
+    auto grads = [&](int i, Real& px, Real& py, Real& rx, Real& ry, Real& rti) {
+        tile_grads<Real>(S.G, S.rt, i, tx + 1, ty + 1, 0, sten, px, py, rx, ry, rti);
+    };
     if (lagged >= 0 ? lagged != 0 : A.lagged != 0) {  // F(t - 1), copied by prefetch_force
         asm volatile("cp.async.wait_all;\n" ::: "memory");
         const Real Fpx = S.Fl[0][ty][tx], Fpy = S.Fl[1][ty][tx];
-        phase3_core<NC, !MOMENTS, STD, true, Real>(m, sten, S.G, S.rt, tx + 1, ty + 1, 0, rho, jx, jy, geth, Fpx,
-                                                   Fpy, store, Ftx, Fty, ux, uy);
+        phase3_core<NC, !MOMENTS, STD, true, Real>(m, grads, rho, jx, jy, geth, Fpx, Fpy, store, Ftx, Fty, ux, uy);
     } else {
-        phase3_core<NC, !MOMENTS, STD, false, Real>(m, sten, S.G, S.rt, tx + 1, ty + 1, 0, rho, jx, jy, geth,
-                                                    Real(0), Real(0), store, Ftx, Fty, ux, uy);
+        phase3_core<NC, !MOMENTS, STD, false, Real>(m, grads, rho, jx, jy, geth, Real(0), Real(0), store, Ftx, Fty, ux,
+                                                    uy);
     }
     if constexpr (MOMENTS) {
 #pragma unroll
@@ -1148,6 +1166,7 @@ template <int NC, int ST, int TY, bool MOMENTS, bool STD = false, bool SPEC = fa
 // compiler chooses.
 __global__ void __launch_bounds__(kTX* TY, ST == ST_F64 ? 1 : (kParkLast<NC, ST, TY> ? 5 : 1024 / (kTX * TY)))
     fused_step(StepArgs A, Planes P) {
+    pdl_wait();
     using Real = typename StoreTraits<ST>::Real;
     constexpr bool PARK = kParkLast<NC, ST, TY>;
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -31,6 +31,23 @@ inline cudaError_t ensure_smem_attr(std::atomic<unsigned long long>& done, const
         if (e_ != cudaSuccess) return e_;                                                  \
     } while (0)
 
+// A launch, programmatic behind the stream's preceding launch if pdl (only for kernels that call
+// pdl_wait before they touch memory).
+template <typename... P, typename... Q>
+cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl, Q&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, static_cast<Q&&>(args)...);
+}
+
 // Tile heights of the fused step (tile width is one warp).  The host picks one per
 // lattice (fmlbm_set_tile_height / the batch autotuner).
 constexpr int kTileYSmall = 8;
@@ -117,8 +134,7 @@ inline bool spec_options(const StepArgs& A) {
         dim3 grid((A.nx + kTX - 1) / kTX, (A.ny + TY - 1) / TY);                                          \
         const Planes P = make_planes(A, NC, kDev16<ST>,                                                   \
                                      ST == ST_F64 ? 8 : (ST == ST_F32 ? 4 : 2));                          \
-        k<<<grid, dim3(kTX, TY), smem, s>>>(A, P);                                                        \
-        return cudaGetLastError();                                                                        \
+        return launch_kernel(k, grid, dim3(kTX, TY), smem, s, A.pdl != 0, A, P);                          \
     }                                                                                                     \
     template <int NC>                                                                                     \
     static cudaError_t launch_step_ty_##ST(const StepArgs& A, bool moments, int tile_y, cudaStream_t s) { \

@@ -284,8 +284,10 @@ __global__ void __launch_bounds__(kTX* TY, NPARK > 0 ? 4 : 3) fused_step_pair(St
             if (valid1) store_gp<ST>(P, i, a, node0 + kTX, v.y);
         };
         V Ftx, Fty, ux, uy;
-        phase3_core<NC, true, false, LAG, V>(m, A.stencil, S.G, S.rt, tx + 1, ty + 1, 0, r, jx, jy, geth, Fpx, Fpy,
-                                             store, Ftx, Fty, ux, uy);
+        auto grads = [&](int i, V& px, V& py, V& rx, V& ry, V& rti) {
+            tile_grads<V>(S.G, S.rt, i, tx + 1, ty + 1, 0, A.stencil, px, py, rx, ry, rti);
+        };
+        phase3_core<NC, true, false, LAG, V>(m, grads, r, jx, jy, geth, Fpx, Fpy, store, Ftx, Fty, ux, uy);
         float* Fout = static_cast<float*>(A.Fout);
         Fout[node0] = Ftx.x;
         Fout[nxy + node0] = Fty.x;
