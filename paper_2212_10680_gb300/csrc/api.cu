@@ -64,6 +64,7 @@ struct fmlbm_handle {
     bool owns_buffers = true;        // false: g, g0 and F belong to the caller (fmlbm_create_with_buffers)
     long long wait_polls = kMaxPolls;  // bound of a wait for a tile copy (bulk-copy step forms)
     int check_y0 = 0, check_y1 = 0;    // rows the domain check covers (check_y1 = 0: all)
+    void* fields = nullptr;            // split step: scratch planes (null: the step runs fused)
     long long* done = nullptr;         // per-tile step counters of the multi-step kernel
     CUtensorMap tmap[2][2];          // [buffer][0: float planes, 1: 16-bit planes]
     std::string last_error;
@@ -199,6 +200,7 @@ StepArgs make_args(const fmlbm_handle* h, int src) {
     A.Fout = h->F[src ^ 1];
     A.err = h->err_dev;
     A.wait_polls = h->wait_polls;
+    A.fields = h->fields;
     A.check_y0 = h->check_y0;
     A.check_y1 = h->check_y1;
     MixConst mc = h->mc;
@@ -405,6 +407,7 @@ void release(fmlbm_handle* h) {
     if (h->rho_prev) cudaFree(h->rho_prev);
     if (h->partial) cudaFree(h->partial);
     if (h->done) cudaFree(h->done);
+    if (h->fields) cudaFree(h->fields);
     if (h->diag_dev) cudaFree(h->diag_dev);
     if (h->diag_host) cudaFreeHost(h->diag_host);
     for (int k = 0; k < kDiagSlots; ++k)
@@ -594,6 +597,14 @@ fmlbm_status create_handle(const fmlbm_mixture* mixture, const fmlbm_lattice* la
         return FMLBM_E_CUDA;
     }
     cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
+    // the split step's planes; without them (no memory left) the lattice steps fused
+    const bool f64 = lattice->precision == FMLBM_FP64;
+    if ((f64 || lattice->precision == FMLBM_FP16DEV_LNF64 || lattice->precision == FMLBM_BF16DEV_LNF64) &&
+        lattice->formulation == FMLBM_WELL_BALANCED &&
+        cudaMalloc(&h->fields, split_planes(h->nc, f64) * nxy * real_size(lattice->precision)) != cudaSuccess) {
+        cudaGetLastError();
+        h->fields = nullptr;
+    }
     setup_tma(h);
     *out = h;
     return FMLBM_OK;
@@ -783,6 +794,7 @@ fmlbm_status fmlbm_step(fmlbm_handle* h, int64_t nsteps) {
         StepArgs A = make_args(h, h->cur);
         const int64_t fused = h->pending;
         A.pdl = pdl && fused < 0;
+        A.pdl_chain = pdl;
         if (fused >= 0) {  // this step also reduces the state it reads
             A.diag_partial = partial_set(h, fused);
             A.rho_prev = h->rho_prev;

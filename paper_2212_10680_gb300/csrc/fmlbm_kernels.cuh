@@ -138,10 +138,13 @@ struct StepArgs {
     void* diag_partial;
     void* rho_prev;  // [N][ny][nx] in the storage arithmetic type
     int have_prev;
+    void* fields;    // split step: scratch planes [split_planes][ny][nx] of the arithmetic type
     // rows [check_y0, check_y1) whose nodes the domain check covers (check_y1 = 0: all); a slab
     // of a decomposed lattice leaves out its ghost rows, whose update is discarded
     int check_y0, check_y1;
     int pdl;               // host: launch programmatically behind the stream's preceding launch
+    int pdl_chain;         // host: a step of several launches may chain them programmatically
+    int pad0;
     long long wait_polls;  // polls of a bounded wait for a tile copy (bulk-copy step forms)
 };
 __device__ __forceinline__ bool checked_row(const StepArgs& A, int y) {

@@ -6,6 +6,7 @@
 
 #include "fmlbm_multi.cuh"
 #include "fmlbm_pair.cuh"
+#include "fmlbm_split.cuh"
 #include "fmlbm_tma.cuh"
 
 namespace fmlbm {
@@ -122,6 +123,32 @@ inline bool spec_options(const StepArgs& A) {
     return A.mixd.eos == 0 && A.stencil == 0 && A.lagged != 0 && A.standard == 0;
 }
 
+// The split step (fmlbm_split.cuh), TY rows per block of both launches.
+template <int NC, int ST, int TY>
+cudaError_t launch_split_ty(const StepArgs& A, cudaStream_t s) {
+    using Real = typename StoreTraits<ST>::Real;
+    const dim3 block(kTX, TY), grid((A.nx + kTX - 1) / kTX, (A.ny + TY - 1) / TY);
+    cudaError_t e;
+    if (A.diag_partial != nullptr) {  // the sums go by 32 x 8 strips
+        auto k = node_fields<NC, ST, kRedTY, true>;
+        constexpr size_t smem = (size_t)NC * kRedTY * kTX * sizeof(Real);
+        e = launch_kernel(k, dim3(grid.x, (A.ny + kRedTY - 1) / kRedTY), dim3(kTX, kRedTY), smem, s, A.pdl != 0, A);
+    } else {
+        e = launch_kernel(node_fields<NC, ST, TY, false>, grid, block, 0, s, A.pdl != 0, A);
+    }
+    if (e != cudaSuccess) return e;
+    auto k = collide_fields<NC, ST, TY>;
+    constexpr size_t smem = sizeof(StepSmem<Real, NC, TY>);
+    FMLBM_ENSURE_SMEM(k, smem);
+    return launch_kernel(k, grid, block, smem, s, A.pdl != 0 || A.pdl_chain != 0, A);
+}
+template <int NC, int ST>
+cudaError_t launch_split(const StepArgs& A, cudaStream_t s) {
+    // Two-row blocks spread a small lattice over the multiprocessors; above 2^16 nodes there are
+    // more 8-row blocks than multiprocessors and the smaller halo counts.
+    return (size_t)A.nx * A.ny <= 65536 ? launch_split_ty<NC, ST, 2>(A, s) : launch_split_ty<NC, ST, 8>(A, s);
+}
+
 #define FMLBM_DEFINE_LAUNCHERS(ST)                                                                        \
     template <int NC, bool MOM, int TY, bool STD = false, bool SPEC = false>                              \
     static cudaError_t launch_step_nc_##ST(const StepArgs& A, cudaStream_t s) {                           \
@@ -145,6 +172,9 @@ inline bool spec_options(const StepArgs& A) {
                                : launch_step_nc_##ST<NC, false, kTileYSmall, true>(A, s);                 \
         } else {                                                                                          \
             if (A.standard) return cudaErrorNotSupported;                                                 \
+        }                                                                                                 \
+        if constexpr (kSplitStep<ST>) {                                                                   \
+            if (!moments && A.fields != nullptr && tile_y == kTileYSmall) return launch_split<NC, ST>(A, s); \
         }                                                                                                 \
         if (tile_y == kTileYLarge)                                                                        \
             return moments ? launch_step_nc_##ST<NC, true, kTileYLarge>(A, s)                             \
