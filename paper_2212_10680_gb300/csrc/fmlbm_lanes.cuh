@@ -9,11 +9,14 @@
 // kernel, the one-node kernels, the bulk-copy kernels and the batch kernel agree bit for
 // bit.  Where the arithmetic wants a fused multiply-add it says so (vfma).
 //
-// Reciprocal and logarithm work per lane: the exact library forms in double, the
-// hardware approximations in float (below), well inside the FP32 error budget.
+// Reciprocal and logarithm work per lane: in double the IEEE division and the integer logarithm
+// of fmlbm_log.cuh, in float the hardware approximations (below), well inside the FP32 error
+// budget.
 #pragma once
 
 #include <cuda_runtime.h>
+
+#include "fmlbm_log.cuh"
 
 namespace fmlbm {
 
@@ -72,7 +75,7 @@ __device__ __forceinline__ float sln(float x) {
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l2) : "f"(x));
     return __fmul_rn(l2, 0.693147180559945309f);  // ln 2
 }
-__device__ __forceinline__ double sln(double x) { return log(x); }
+__device__ __forceinline__ double sln(double x) { return ln_f64(x); }
 __device__ __forceinline__ float slog1p(float x) { return log1pf(x); }
 __device__ __forceinline__ double slog1p(double x) { return log1p(x); }
 
