@@ -201,6 +201,7 @@ StepArgs make_args(const fmlbm_handle* h, int src) {
     A.err = h->err_dev;
     A.wait_polls = h->wait_polls;
     A.fields = h->fields;
+    A.sms = h->sms;
     A.check_y0 = h->check_y0;
     A.check_y1 = h->check_y1;
     MixConst mc = h->mc;

@@ -144,7 +144,7 @@ struct StepArgs {
     int check_y0, check_y1;
     int pdl;               // host: launch programmatically behind the stream's preceding launch
     int pdl_chain;         // host: a step of several launches may chain them programmatically
-    int pad0;
+    int sms;               // host: multiprocessors of the device
     long long wait_polls;  // polls of a bounded wait for a tile copy (bulk-copy step forms)
 };
 __device__ __forceinline__ bool checked_row(const StepArgs& A, int y) {
@@ -717,6 +717,67 @@ __device__ __forceinline__ void phase2(const MixConstT<Real>& m, StepSmem<Real, 
             phase2_core<NC, Real>(m, S.rt, S.lf, S.G, stencil, kTX + (e & 1), e >> 1, 0);
 }
 
+// Collision g' = g - omega (g - g^eq) + fcoef F_a, with g^eq of Eq. eqLBEMCb (rho_0 = 0)
+// and F_a of Eq. eqLBEMCfinal3, evaluated for each pair of opposite directions
+// (e_abar = -e_a): the parts even in e are shared, the odd parts change sign.
+//   g^eq_a = w rho [3 eu + 4.5 eu^2 - 1.5 u^2]
+//   F_a    = w [3 eF - 3 uF + 9 eu eF + (c_a - 1) ug + 3 eu eg],  c_a = (3 e^2 - 2)/2
+// (eu = e_a.u, eF = e_a.F_i, eg = e_a.grad rho_i, uF = u.F_i, ug = u.grad rho_i).  With
+// rw = omega rho_i, fc = fcoef, base = 1.5 rw u^2 the post-collision value is
+//   g'_a = (1 - omega) g_a + even_a + odd_a,   g'_abar = (1 - omega) g_abar + even_a - odd_a
+//   even_a = w_a [eu (e_a.V) + cb_a],  V = 4.5 rw u + fc (9 F_i + 3 grad rho_i),
+//            cb_a = fc (c_a - 1) ug - 3 fc uF - base
+//   odd_a  = 3 w_a (rw eu + fc eF) = e_a.O (axes), e_a.O / 4 (diagonals),
+//            O = (rw u + fc F_i) / 3
+//   g'_0   = (1 - omega) g_0 + rw + (4/9) (-base - 3 fc uF - 2 fc ug)
+// and each e_a.X is written out (components 0, +-1): no multiplication by zero.
+template <bool STD, typename V, typename E, typename Store>
+__device__ __forceinline__ void collide_node(const MixConstT<E>& m, const V (&h)[9], V rho, V ux, V uy, V Fx, V Fy,
+                                             V grx, V gry, Store&& store) {
+    const E fc = m.fcoef;
+    const V usq15 = vmul(vbc<V>(E(1.5)), vfma(ux, ux, vmul(uy, uy)));
+    const V rw = vmul(vbc<V>(m.omega), rho);
+    const V uF = vfma(ux, Fx, vmul(uy, Fy));
+    const V a0 = vneg(vfma(rw, usq15, vmul(vbc<V>(E(3) * fc), uF)));  // -base - 3 fc uF
+    V cb_ax, cb_dg, Vx, Vy, g0c;
+    if constexpr (STD) {
+        // the forcing term's grad rho_i part belongs to the well-balanced scheme only;
+        // the standard equilibrium adds w_a rho_i (a != 0) and w_0 rho_i (a = 0)
+        cb_ax = vadd(a0, rw);
+        cb_dg = cb_ax;
+        Vx = vfma(vbc<V>(E(4.5)), vmul(rw, ux), vmul(vbc<V>(E(9) * fc), Fx));
+        Vy = vfma(vbc<V>(E(4.5)), vmul(rw, uy), vmul(vbc<V>(E(9) * fc), Fy));
+        g0c = vmul(vbc<V>(E(4.0 / 9.0)), vadd(rw, a0));
+    } else {
+        const V ug = vfma(ux, grx, vmul(uy, gry));
+        cb_ax = vfma(vbc<V>(E(-0.5) * fc), ug, a0);
+        cb_dg = vfma(vbc<V>(fc), ug, a0);
+        Vx = vfma(vbc<V>(E(4.5)), vmul(rw, ux), vfma(vbc<V>(E(9) * fc), Fx, vmul(vbc<V>(E(3) * fc), grx)));
+        Vy = vfma(vbc<V>(E(4.5)), vmul(rw, uy), vfma(vbc<V>(E(9) * fc), Fy, vmul(vbc<V>(E(3) * fc), gry)));
+        g0c = vfma(vbc<V>(E(4.0 / 9.0)), vfma(vbc<V>(E(-2) * fc), ug, a0), rw);
+    }
+    const V rw3 = vmul(rw, vbc<V>(E(1.0 / 3.0)));
+    const V fc_3 = vbc<V>(fc * E(1.0 / 3.0));
+    const V Ox = vfma(rw3, ux, vmul(fc_3, Fx));
+    const V Oy = vfma(rw3, uy, vmul(fc_3, Fy));
+    const V keep = vbc<V>(E(1) - m.omega);
+    const V w1 = vbc<V>(E(1.0 / 9.0)), w5 = vbc<V>(E(1.0 / 36.0)), quarter = vbc<V>(E(0.25));
+    // g'_a = keep g_a + (w_a X_a +- odd_a), X_a = eu (e_a.V) + cb_a: one fused product each
+    store(0, vfma(keep, h[0], g0c));
+    const V X1 = vfma(ux, Vx, cb_ax);
+    store(1, vfma(keep, h[1], vfma(w1, X1, Ox)));
+    store(3, vfma(keep, h[3], vfma(w1, X1, vneg(Ox))));
+    const V X2 = vfma(uy, Vy, cb_ax);
+    store(2, vfma(keep, h[2], vfma(w1, X2, Oy)));
+    store(4, vfma(keep, h[4], vfma(w1, X2, vneg(Oy))));
+    const V X5 = vfma(vadd(ux, uy), vadd(Vx, Vy), cb_dg), o5 = vmul(quarter, vadd(Ox, Oy));
+    store(5, vfma(keep, h[5], vfma(w5, X5, o5)));
+    store(7, vfma(keep, h[7], vfma(w5, X5, vneg(o5))));
+    const V X6 = vfma(vsub(uy, ux), vsub(Vy, Vx), cb_dg), o6 = vmul(quarter, vsub(Oy, Ox));
+    store(6, vfma(keep, h[6], vfma(w5, X6, o6)));
+    store(8, vfma(keep, h[8], vfma(w5, X6, vneg(o6))));
+}
+
 // Phase 3 at one lane of nodes: force (step 7), velocity (step 1), equilibrium and
 // forcing (step 8) and collision (step 9).
 //   grads(i, px, py, rx, ry, rti): the gradients of Phi_i and of rho~_i at the node, and rho~_i;
@@ -756,65 +817,10 @@ __device__ __forceinline__ void phase3_core(const MixConstT<E>& m, Grads&& grads
     for (int i = 1; i < NC; ++i) rho_t = vadd(rho_t, rho[i]);
     const V half = vbc<V>(E(0.5));
     const V inv_rho = vrcp(rho_t);
-    // Collision g' = g - omega (g - g^eq) + fcoef F_a, with g^eq of Eq. eqLBEMCb (rho_0 = 0)
-    // and F_a of Eq. eqLBEMCfinal3, evaluated for each pair of opposite directions
-    // (e_abar = -e_a): the parts even in e are shared, the odd parts change sign.
-    //   g^eq_a = w rho [3 eu + 4.5 eu^2 - 1.5 u^2]
-    //   F_a    = w [3 eF - 3 uF + 9 eu eF + (c_a - 1) ug + 3 eu eg],  c_a = (3 e^2 - 2)/2
-    // (eu = e_a.u, eF = e_a.F_i, eg = e_a.grad rho_i, uF = u.F_i, ug = u.grad rho_i).  With
-    // rw = omega rho_i, fc = fcoef, base = 1.5 rw u^2 the post-collision value is
-    //   g'_a = (1 - omega) g_a + even_a + odd_a,   g'_abar = (1 - omega) g_abar + even_a - odd_a
-    //   even_a = w_a [eu (e_a.V) + cb_a],  V = 4.5 rw u + fc (9 F_i + 3 grad rho_i),
-    //            cb_a = fc (c_a - 1) ug - 3 fc uF - base
-    //   odd_a  = 3 w_a (rw eu + fc eF) = e_a.O (axes), e_a.O / 4 (diagonals),
-    //            O = (rw u + fc F_i) / 3
-    //   g'_0   = (1 - omega) g_0 + rw + (4/9) (-base - 3 fc uF - 2 fc ug)
-    // and each e_a.X is written out (components 0, +-1): no multiplication by zero.
     auto collide = [&](int i, V Fx, V Fy, V grx, V gry) {
-        const E fc = m.fcoef;
-        const V usq15 = vmul(vbc<V>(E(1.5)), vfma(ux, ux, vmul(uy, uy)));
         V h[9];
         geth(i, h);
-        const V rw = vmul(vbc<V>(m.omega), rho[i]);
-        const V uF = vfma(ux, Fx, vmul(uy, Fy));
-        const V a0 = vneg(vfma(rw, usq15, vmul(vbc<V>(E(3) * fc), uF)));  // -base - 3 fc uF
-        V cb_ax, cb_dg, Vx, Vy, g0c;
-        if constexpr (STD) {
-            // the forcing term's grad rho_i part belongs to the well-balanced scheme only;
-            // the standard equilibrium adds w_a rho_i (a != 0) and w_0 rho_i (a = 0)
-            cb_ax = vadd(a0, rw);
-            cb_dg = cb_ax;
-            Vx = vfma(vbc<V>(E(4.5)), vmul(rw, ux), vmul(vbc<V>(E(9) * fc), Fx));
-            Vy = vfma(vbc<V>(E(4.5)), vmul(rw, uy), vmul(vbc<V>(E(9) * fc), Fy));
-            g0c = vmul(vbc<V>(E(4.0 / 9.0)), vadd(rw, a0));
-        } else {
-            const V ug = vfma(ux, grx, vmul(uy, gry));
-            cb_ax = vfma(vbc<V>(E(-0.5) * fc), ug, a0);
-            cb_dg = vfma(vbc<V>(fc), ug, a0);
-            Vx = vfma(vbc<V>(E(4.5)), vmul(rw, ux), vfma(vbc<V>(E(9) * fc), Fx, vmul(vbc<V>(E(3) * fc), grx)));
-            Vy = vfma(vbc<V>(E(4.5)), vmul(rw, uy), vfma(vbc<V>(E(9) * fc), Fy, vmul(vbc<V>(E(3) * fc), gry)));
-            g0c = vfma(vbc<V>(E(4.0 / 9.0)), vfma(vbc<V>(E(-2) * fc), ug, a0), rw);
-        }
-        const V rw3 = vmul(rw, vbc<V>(E(1.0 / 3.0)));
-        const V fc_3 = vbc<V>(fc * E(1.0 / 3.0));
-        const V Ox = vfma(rw3, ux, vmul(fc_3, Fx));
-        const V Oy = vfma(rw3, uy, vmul(fc_3, Fy));
-        const V keep = vbc<V>(E(1) - m.omega);
-        const V w1 = vbc<V>(E(1.0 / 9.0)), w5 = vbc<V>(E(1.0 / 36.0)), quarter = vbc<V>(E(0.25));
-        // g'_a = keep g_a + (w_a X_a +- odd_a), X_a = eu (e_a.V) + cb_a: one fused product each
-        store(i, 0, vfma(keep, h[0], g0c));
-        const V X1 = vfma(ux, Vx, cb_ax);
-        store(i, 1, vfma(keep, h[1], vfma(w1, X1, Ox)));
-        store(i, 3, vfma(keep, h[3], vfma(w1, X1, vneg(Ox))));
-        const V X2 = vfma(uy, Vy, cb_ax);
-        store(i, 2, vfma(keep, h[2], vfma(w1, X2, Oy)));
-        store(i, 4, vfma(keep, h[4], vfma(w1, X2, vneg(Oy))));
-        const V X5 = vfma(vadd(ux, uy), vadd(Vx, Vy), cb_dg), o5 = vmul(quarter, vadd(Ox, Oy));
-        store(i, 5, vfma(keep, h[5], vfma(w5, X5, o5)));
-        store(i, 7, vfma(keep, h[7], vfma(w5, X5, vneg(o5))));
-        const V X6 = vfma(vsub(uy, ux), vsub(Vy, Vx), cb_dg), o6 = vmul(quarter, vsub(Oy, Ox));
-        store(i, 6, vfma(keep, h[6], vfma(w5, X6, o6)));
-        store(i, 8, vfma(keep, h[8], vfma(w5, X6, vneg(o6))));
+        collide_node<STD, V, E>(m, h, rho[i], ux, uy, Fx, Fy, grx, gry, [&](int a, V v) { store(i, a, v); });
     };
     if constexpr (LAG) {
         ux = vmul(vfma(half, Fpx, jx), inv_rho);

@@ -4,7 +4,9 @@
 
 #include <atomic>
 
+#include "fmlbm_march.cuh"
 #include "fmlbm_multi.cuh"
+#include "fmlbm_pack.cuh"
 #include "fmlbm_pair.cuh"
 #include "fmlbm_split.cuh"
 #include "fmlbm_tma.cuh"
@@ -149,6 +151,37 @@ cudaError_t launch_split(const StepArgs& A, cudaStream_t s) {
     return (size_t)A.nx * A.ny <= 65536 ? launch_split_ty<NC, ST, 2>(A, s) : launch_split_ty<NC, ST, 8>(A, s);
 }
 
+// The packed step, two components, five blocks per multiprocessor (48 registers).
+template <int NC, int ST, bool SPEC>
+cudaError_t launch_pack(const StepArgs& A, cudaStream_t s) {
+    auto k = pack_step<NC, ST, SPEC, 5>;
+    constexpr size_t smem = pack_smem_bytes<NC>();
+    FMLBM_ENSURE_SMEM(k, smem);
+    const dim3 grid((A.nx + kTX - 1) / kTX, (A.ny + kTileYSmall - 1) / kTileYSmall);
+    const Planes P = make_planes(A, NC, kDev16<ST>, ST == ST_F32 ? 4 : 2);
+    return launch_kernel(k, grid, dim3(kTX, kTileYSmall), smem, s, A.pdl != 0, A, P);
+}
+
+// The marching step: 16 (two components) or 12 (three) warps per multiprocessor.
+template <int NC, int ST, bool SPEC, bool NOALLOC>
+cudaError_t launch_march_as(const StepArgs& A, cudaStream_t s) {
+    constexpr int MINB = NC == 2 ? 4 : 3;
+    auto k = march_step<NC, ST, SPEC, NOALLOC, MINB>;
+    constexpr size_t smem = march_smem_bytes<NC>();
+    FMLBM_ENSURE_SMEM(k, smem);
+    const int strips = (A.nx + kMarchCols - 1) / kMarchCols;
+    const int chunk = march_chunk_rows(A.ny, strips, A.sms * MINB * kMarchWarps);
+    const int warps = strips * ((A.ny + chunk - 1) / chunk);
+    const Planes P = make_planes(A, NC, kDev16<ST>, ST == ST_F32 ? 4 : 2);
+    return launch_kernel(k, dim3((warps + kMarchWarps - 1) / kMarchWarps), dim3(32 * kMarchWarps), smem, s, A.pdl != 0, A,
+                         P, strips, chunk);
+}
+template <int NC, int ST, bool SPEC>
+cudaError_t launch_march(const StepArgs& A, cudaStream_t s) {
+    return march_state_bytes<NC, ST>(A) <= kMarchL2Bytes ? launch_march_as<NC, ST, SPEC, true>(A, s)
+                                                         : launch_march_as<NC, ST, SPEC, false>(A, s);
+}
+
 #define FMLBM_DEFINE_LAUNCHERS(ST)                                                                        \
     template <int NC, bool MOM, int TY, bool STD = false, bool SPEC = false>                              \
     static cudaError_t launch_step_nc_##ST(const StepArgs& A, cudaStream_t s) {                           \
@@ -180,6 +213,14 @@ cudaError_t launch_split(const StepArgs& A, cudaStream_t s) {
             return moments ? launch_step_nc_##ST<NC, true, kTileYLarge>(A, s)                             \
                            : launch_step_nc_##ST<NC, false, kTileYLarge>(A, s);                           \
         if (tile_y == kTileYHuge && !moments) return launch_step_nc_##ST<NC, false, kTileYHuge>(A, s);    \
+        if constexpr (kSpecStep<ST> && (NC == 2 || NC == 3)) {                                            \
+            if (!moments && A.diag_partial == nullptr && march_applies<NC, ST>(A))                        \
+                return spec_options(A) ? launch_march<NC, ST, true>(A, s) : launch_march<NC, ST, false>(A, s); \
+        }                                                                                                 \
+        if constexpr (kSpecStep<ST> && NC == 2) {                                                         \
+            if (!moments && (size_t)A.nx * A.ny >= kPackNodes)                                            \
+                return spec_options(A) ? launch_pack<NC, ST, true>(A, s) : launch_pack<NC, ST, false>(A, s); \
+        }                                                                                                 \
         if constexpr (kSpecStep<ST>) {                                                                    \
             if (!moments && spec_options(A)) return launch_step_nc_##ST<NC, false, kTileYSmall, false, true>(A, s); \
         }                                                                                                 \
