@@ -214,7 +214,7 @@ cudaError_t launch_march(const StepArgs& A, cudaStream_t s) {
                            : launch_step_nc_##ST<NC, false, kTileYLarge>(A, s);                           \
         if (tile_y == kTileYHuge && !moments) return launch_step_nc_##ST<NC, false, kTileYHuge>(A, s);    \
         if constexpr (kSpecStep<ST> && (NC == 2 || NC == 3)) {                                            \
-            if (!moments && A.diag_partial == nullptr && march_applies<NC, ST>(A))                        \
+            if (!moments && A.diag_partial == nullptr && march_applies(A))                                \
                 return spec_options(A) ? launch_march<NC, ST, true>(A, s) : launch_march<NC, ST, false>(A, s); \
         }                                                                                                 \
         if constexpr (kSpecStep<ST> && NC == 2) {                                                         \

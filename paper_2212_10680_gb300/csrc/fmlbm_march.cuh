@@ -6,9 +6,11 @@
 // (steps 7-9): the three rows a stencil reads are rolling registers of the lane that owns the
 // column, the neighbours in x come from the adjacent lanes by shuffles.  The pulled values wait in
 // shared memory for the two rows between their sums and their collision (each lane reads back its
-// own values, so there is no barrier), and the loads of the next row are issued as soon as the
-// row's values are parked, in flight during the row's arithmetic.  Two components share a packed
-// value (fmlbm_comps.cuh).
+// own values, so there is no barrier; only they are parked, the sums are formed again: with the row
+// sums and gradients beside them, 4096^2 ternary FP32 took 803 us instead of 760, as what a block
+// parks is taken from the L1), and the loads of the next row are issued as soon as the row's values
+// are parked, in flight during the row's arithmetic.  Two components share a packed value
+// (fmlbm_comps.cuh).
 //
 // The tile step is bound by its blocks' phases: every block loads, then computes (6,000 of 14,700
 // cycles of a block pass until its loads have come), its instructions (816 per node, binary FP32)
@@ -30,30 +32,25 @@ namespace fmlbm {
 
 constexpr int kMarchCols = 28;  // columns a strip owns
 
-// Where the marching step is the faster one (GB300, us per step, tile step -> marching step):
-//   two components   768^2 FP32 19.6 -> 18.0, 1024^2 37.5 -> 30.4, 1536^2 78.0 -> 75.9, 2048^2 136 -> 134;
-//                    FP16 768^2 17.1 -> 16.8, 1024^2 30.1 -> 27.9, 2048^2 111 -> 104, 4096^2 433 -> 417
-//   three components 768^2 FP32 33.3 -> 26.1, 1024^2 55.4 -> 49.7, 2048^2 201 -> 199, 4096^2 795 -> 803;
-//                    BF16 768^2 26.1 -> 22.9, 1024^2 44.9 -> 38.1, 2048^2 166 -> 155, 4096^2 660 -> 639
+// Where the marching step is the faster one (GB300, us per step, packed or tile step -> marching):
+//   two components   768^2 FP32 19.6 -> 18.2, 1024^2 37.0 -> 31.0, 2048^2 132 -> 130;
+//                    FP16 768^2 17.1 -> 16.8, 1024^2 29.9 -> 28.7, 2048^2 111 -> 104, 4096^2 433 -> 417
+//   three components 768^2 FP32 33.3 -> 26.1, 1024^2 55.4 -> 50.0, 2048^2 201 -> 195, 4096^2 795 -> 760;
+//                    BF16 768^2 26.1 -> 22.9, 1024^2 44.9 -> 38.1, 2048^2 165 -> 157, 4096^2 657 -> 619
 // Below 2^19 nodes a chunk has so few rows that its four halo rows outweigh the rest (512^2 FP32
-// 9.2 -> 9.8); FP32 states of more than 256 MB are bound by DRAM either way, and the tiles' row
-// order reads it more evenly.
+// 9.2 -> 9.8).
 constexpr size_t kMarchNodes = 1 << 19;
-constexpr size_t kMarchF32Bytes = 256u << 20;
 // States up to this size stay in the 129 MB L2 from the step that writes them to the step that
 // reads them; their loads then go without a place in L1, whose turnover cost more than its hits
-// gave (1024^2 binary FP32 36.2 -> 30.4 us, 1280^2 FP16 43.7 -> 40.5).  From DRAM the sector-wise
-// requests are slower (2048^2 FP32 134 -> 157).
+// gave (1024^2 binary FP32 35.9 -> 31.0 us, 1280^2 FP16 43.7 -> 40.5).  From DRAM the sector-wise
+// requests are slower (2048^2 FP32 130 -> 157).
 constexpr size_t kMarchL2Bytes = 125000000;
 
 template <int NC, int ST>
 inline size_t march_state_bytes(const StepArgs& A) {  // distributions and stored force a step reads
     return (size_t)A.nx * A.ny * (ST == ST_F32 ? NC * 36 + 8 : NC * 20 + 8);
 }
-template <int NC, int ST>
-inline bool march_applies(const StepArgs& A) {
-    return (size_t)A.nx * A.ny >= kMarchNodes && (ST != ST_F32 || march_state_bytes<NC, ST>(A) <= kMarchF32Bytes);
-}
+inline bool march_applies(const StepArgs& A) { return (size_t)A.nx * A.ny >= kMarchNodes; }
 // Rows per chunk: all warps resident at once (one wave of `capacity` warps) while that keeps a
 // chunk below 96 rows; otherwise as many waves as bring it there (4096^2 BF16 binary, 256 rows in
 // one wave 529 us, 125 rows in two 416 us).
@@ -66,14 +63,12 @@ inline int march_chunk_rows(int ny, int strips, int capacity) {
 
 constexpr int kMarchWarps = 4;  // warps (neighbouring strips) per block
 
-// 16-byte vectors a lane parks per row: the first moment, the densities and the pulled values;
-// then, an iteration later, grad rho~.
-template <int NC> constexpr int kParkVecs = (10 * NC + 2 + 3) / 4;
-template <int NC> constexpr int kGradVecs = (2 * NC + 3) / 4;
-template <int NC> constexpr int kSlotVecs = (kParkVecs<NC> + kGradVecs<NC>) * 32;
+// Words a lane parks per row: the pulled values (their sums are formed again at the collision:
+// what a block parks is taken from the L1, whose size the step feels).
+template <int NC> constexpr int kParkWords = 9 * NC;
 template <int NC>
 constexpr size_t march_smem_bytes() {
-    return (size_t)kMarchWarps * 3 * kSlotVecs<NC> * 16;
+    return (size_t)kMarchWarps * 3 * kParkWords<NC> * 32 * sizeof(float);
 }
 
 // East and west neighbours of a value held by every lane (lane l of the warp: column l).  The
@@ -113,19 +108,29 @@ __device__ __forceinline__ void grad_rows(V cn, V cs, V sn, V ss, V dn, V dc, V 
     }
 }
 
-// Q vectors of a lane's words to and from its place in a slot.
-template <int Q>
-__device__ __forceinline__ void park_put(float4* slot, int lane, const float (&w)[4 * Q]) {
+// A lane's W words to and from a slot: 16-byte vectors, then an 8-byte and a 4-byte remainder.
+template <int W>
+__device__ __forceinline__ void park_put(float* slot, int lane, const float (&w)[W]) {
 #pragma unroll
-    for (int q = 0; q < Q; ++q) slot[q * 32 + lane] = make_float4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+    for (int q = 0; q < W / 4; ++q)
+        reinterpret_cast<float4*>(slot)[q * 32 + lane] = make_float4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+    float* rest = slot + (W / 4) * 128;
+    if constexpr (W % 4 >= 2) reinterpret_cast<float2*>(rest)[lane] = make_float2(w[W / 4 * 4], w[W / 4 * 4 + 1]);
+    if constexpr (W % 2 == 1) rest[(W % 4 == 3 ? 64 : 0) + lane] = w[W - 1];
 }
-template <int Q>
-__device__ __forceinline__ void park_get(const float4* slot, int lane, float (&w)[4 * Q]) {
+template <int W>
+__device__ __forceinline__ void park_get(const float* slot, int lane, float (&w)[W]) {
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        const float4 v = slot[q * 32 + lane];
+    for (int q = 0; q < W / 4; ++q) {
+        const float4 v = reinterpret_cast<const float4*>(slot)[q * 32 + lane];
         w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
     }
+    const float* rest = slot + (W / 4) * 128;
+    if constexpr (W % 4 >= 2) {
+        const float2 v = reinterpret_cast<const float2*>(rest)[lane];
+        w[W / 4 * 4] = v.x; w[W / 4 * 4 + 1] = v.y;
+    }
+    if constexpr (W % 2 == 1) w[W - 1] = rest[(W % 4 == 3 ? 64 : 0) + lane];
 }
 
 // The pulled values as loaded: 16-bit values are widened where they are used, so that nothing
@@ -152,7 +157,7 @@ template <> struct MarchRaw<ST_F32> { using T = float; };
 // One strip x chunk: columns x0 .. x0 + 27 (those below nx), rows y0 .. y0 + rows - 1, by one
 // warp.  slots: the warp's three parking slots.
 template <int NC, int ST, bool SPEC, bool NOALLOC>
-__device__ __forceinline__ void march_chunk(const StepArgs& A, const Planes& P, const MixConstT<float>& m, float4* slots,
+__device__ __forceinline__ void march_chunk(const StepArgs& A, const Planes& P, const MixConstT<float>& m, float* slots,
                                             int x0, int y0, int rows) {
     using Elem = typename StoreTraits<ST>::Elem;
     using Raw = typename MarchRaw<ST>::T;
@@ -196,15 +201,14 @@ __device__ __forceinline__ void march_chunk(const StepArgs& A, const Planes& P, 
     float* Fout = static_cast<float*>(A.Fout);
     load_row();
     // rolling rows, indexed by the iteration mod 3: rho~ with its x-sums and x-differences, Phi
-    // likewise (one row behind), ln f of the last row
-    Comps<NC> rt[3], rs[3], rd[3], ph[3], ps[3], pd[3], lf = {};
+    // likewise (one row behind), ln f of the last row, grad rho~ of the row to collide next
+    Comps<NC> rt[3], rs[3], rd[3], ph[3], ps[3], pd[3], lf = {}, gx = {}, gy = {};
     const int T = rows + 4;
     auto row_step = [&](auto kc, int it) {
         constexpr int K = decltype(kc)::value, K1 = (K + 2) % 3, K2 = (K + 1) % 3;  // rows y, y - 1, y - 2
-        // row y = y0 - 2 + it: densities, first moment, rho~ (steps 1-2); park
+        // row y = y0 - 2 + it: densities and rho~ (steps 1-2); park the pulled values
         {
-            float pk[4 * kParkVecs<NC>];
-            float jx, jy;
+            float pk[kParkWords<NC>];
             each_group<NC>([&](auto of) {
                 using V = typename decltype(of)::V;
                 constexpr bool PAIR = std::is_same<V, float2>::value;
@@ -215,26 +219,14 @@ __device__ __forceinline__ void march_chunk(const StepArgs& A, const Planes& P, 
                 for (int a = 0; a < 9; ++a) {
                     if constexpr (PAIR) h[a] = make_float2(pulled(i0, a), pulled(i0 + 1, a));
                     else h[a] = pulled(i0, a);
+                    // direction by direction within the group
+#pragma unroll
+                    for (int l = 0; l < (PAIR ? 2 : 1); ++l) pk[9 * i0 + (PAIR ? 2 * a + l : a)] = fmlbm::lane(h[a], l);
                 }
                 const V r = sum9(h);
-                V jxi, jyi;
-                moment_j(h, true, jxi, jyi);
                 of(rt[K]) = vmul(r, of.of(m.invM));
-#pragma unroll
-                for (int l = 0; l < (PAIR ? 2 : 1); ++l) {
-                    jx = i0 + l == 0 ? fmlbm::lane(jxi, l) : vadd(jx, fmlbm::lane(jxi, l));
-                    jy = i0 + l == 0 ? fmlbm::lane(jyi, l) : vadd(jy, fmlbm::lane(jyi, l));
-                    pk[2 + i0 + l] = fmlbm::lane(r, l);
-                    // the pulled values, direction by direction within the group
-#pragma unroll
-                    for (int a = 0; a < 9; ++a) pk[2 + NC + 9 * i0 + (PAIR ? 2 * a + l : a)] = fmlbm::lane(h[a], l);
-                }
             });
-            pk[0] = jx;
-            pk[1] = jy;
-#pragma unroll
-            for (int q = 10 * NC + 2; q < 4 * kParkVecs<NC>; ++q) pk[q] = 0.f;
-            park_put<kParkVecs<NC>>(slots + K * kSlotVecs<NC>, lane, pk);
+            park_put(slots + K * kParkWords<NC> * 32, lane, pk);
         }
         // the next row's loads go out now, and the force of the row this iteration collides
         if (it + 1 < T) load_row();
@@ -290,36 +282,40 @@ __device__ __forceinline__ void march_chunk(const StepArgs& A, const Planes& P, 
                 of(ps[K]) = vadd(e, w);
                 of(pd[K]) = vsub(e, w);
             });
-            // grad rho~ of row y - 1, parked with that row for its collision in the next iteration
-            {
-                float gr[4 * kGradVecs<NC>];
+            if (it >= 4 && own) {
+                // collision of row y - 2 (steps 7-9): the operations of phase3_core
+                float pk[kParkWords<NC>];
+                park_get(slots + K2 * kParkWords<NC> * 32, lane, pk);
+                const int node = (y0 + it - 4) * nx + xc;
+                auto group_h = [&](auto of, auto (&h)[9]) {
+                    constexpr bool PAIR = std::is_same<typename decltype(of)::V, float2>::value;
+                    int i0 = NC - 1;
+                    if constexpr (PAIR) i0 = 2 * of.k;
 #pragma unroll
-                for (int q = 2 * NC; q < 4 * kGradVecs<NC>; ++q) gr[q] = 0.f;
+                    for (int a = 0; a < 9; ++a) {
+                        if constexpr (PAIR) h[a] = make_float2(pk[9 * i0 + 2 * a], pk[9 * i0 + 2 * a + 1]);
+                        else h[a] = pk[9 * i0 + a];
+                    }
+                };
+                // densities and first moment (step 1)
+                Comps<NC> rho;
+                float jx = 0.f, jy = 0.f, rho_t = 0.f;
                 each_group<NC>([&](auto of) {
                     using V = typename decltype(of)::V;
                     constexpr bool PAIR = std::is_same<V, float2>::value;
                     int i0 = NC - 1;
                     if constexpr (PAIR) i0 = 2 * of.k;
-                    V gx, gy;
-                    grad_rows<V>(of(rt[K]), of(rt[K2]), of(rs[K]), of(rs[K2]), of(rd[K]), of(rd[K1]), of(rd[K2]), stencil,
-                                 gx, gy);
+                    V h[9], jxi, jyi;
+                    group_h(of, h);
+                    of(rho) = sum9(h);
+                    moment_j(h, true, jxi, jyi);
 #pragma unroll
                     for (int l = 0; l < (PAIR ? 2 : 1); ++l) {
-                        gr[2 * i0 + l] = fmlbm::lane(gx, l);
-                        gr[2 * i0 + (PAIR ? 2 : 1) + l] = fmlbm::lane(gy, l);
+                        jx = i0 + l == 0 ? fmlbm::lane(jxi, l) : vadd(jx, fmlbm::lane(jxi, l));
+                        jy = i0 + l == 0 ? fmlbm::lane(jyi, l) : vadd(jy, fmlbm::lane(jyi, l));
+                        rho_t = i0 + l == 0 ? fmlbm::lane(of(rho), l) : vadd(rho_t, fmlbm::lane(of(rho), l));
                     }
                 });
-                park_put<kGradVecs<NC>>(slots + K1 * kSlotVecs<NC> + kParkVecs<NC> * 32, lane, gr);
-            }
-            if (it >= 4 && own) {
-                // collision of row y - 2 (steps 7-9): the operations of phase3_core
-                float pk[4 * kParkVecs<NC>], gr[4 * kGradVecs<NC>];
-                park_get<kParkVecs<NC>>(slots + K2 * kSlotVecs<NC>, lane, pk);
-                park_get<kGradVecs<NC>>(slots + K2 * kSlotVecs<NC> + kParkVecs<NC> * 32, lane, gr);
-                const int node = (y0 + it - 4) * nx + xc;
-                float rho_t = pk[2];
-#pragma unroll
-                for (int i = 1; i < NC; ++i) rho_t = vadd(rho_t, pk[2 + i]);
                 const float inv_rho = vrcp(rho_t);
                 float Ftx = 0.f, Fty = 0.f, ux = 0.f, uy = 0.f;
                 Comps<NC> Fx, Fy;
@@ -328,12 +324,10 @@ __device__ __forceinline__ void march_chunk(const StepArgs& A, const Planes& P, 
                     constexpr bool PAIR = std::is_same<V, float2>::value;
                     int i0 = NC - 1;
                     if constexpr (PAIR) i0 = 2 * of.k;
-                    V px, py, rho;
-                    if constexpr (PAIR) rho = make_float2(pk[2 + i0], pk[3 + i0]);
-                    else rho = pk[2 + i0];
+                    V px, py;
                     grad_rows<V>(of(ph[K]), of(ph[K2]), of(ps[K]), of(ps[K2]), of(pd[K]), of(pd[K1]), of(pd[K2]), stencil,
                                  px, py);
-                    const V rti = vmul(rho, of.of(m.invM));
+                    const V rti = of(rt[K2]);
                     of(Fx) = vmul(rti, px);
                     of(Fy) = vmul(rti, py);
 #pragma unroll
@@ -347,45 +341,37 @@ __device__ __forceinline__ void march_chunk(const StepArgs& A, const Planes& P, 
                     constexpr bool PAIR = std::is_same<V, float2>::value;
                     int i0 = NC - 1;
                     if constexpr (PAIR) i0 = 2 * of.k;
-                    V h[9], rho, grx, gry;
-#pragma unroll
-                    for (int a = 0; a < 9; ++a) {
-                        if constexpr (PAIR) h[a] = make_float2(pk[2 + NC + 9 * i0 + 2 * a], pk[3 + NC + 9 * i0 + 2 * a]);
-                        else h[a] = pk[2 + NC + 9 * i0 + a];
-                    }
-                    if constexpr (PAIR) {
-                        rho = make_float2(pk[2 + i0], pk[3 + i0]);
-                        grx = make_float2(gr[2 * i0], gr[2 * i0 + 1]);
-                        gry = make_float2(gr[2 * i0 + 2], gr[2 * i0 + 3]);
-                    } else {
-                        rho = pk[2 + i0];
-                        grx = gr[2 * i0];
-                        gry = gr[2 * i0 + 1];
-                    }
-                    grx = vmul(grx, of.of(m.M));
-                    gry = vmul(gry, of.of(m.M));
+                    V h[9];
+                    group_h(of, h);
+                    const V grx = vmul(of(gx), of.of(m.M)), gry = vmul(of(gy), of.of(m.M));
                     const V u_x = vbc<V>(ux), u_y = vbc<V>(uy);
-                    collide_node<false, V, float>(m, h, rho, u_x, u_y, of(Fx), of(Fy), grx, gry, [&](int a, V v) {
+                    collide_node<false, V, float>(m, h, of(rho), u_x, u_y, of(Fx), of(Fy), grx, gry, [&](int a, V v) {
 #pragma unroll
                         for (int l = 0; l < (PAIR ? 2 : 1); ++l) store_gp<ST>(P, i0 + l, a, node, fmlbm::lane(v, l));
                     });
                 };
                 if (lagged) {
-                    ux = vmul(vfma(0.5f, Fpx, pk[0]), inv_rho);
-                    uy = vmul(vfma(0.5f, Fpy, pk[1]), inv_rho);
+                    ux = vmul(vfma(0.5f, Fpx, jx), inv_rho);
+                    uy = vmul(vfma(0.5f, Fpy, jy), inv_rho);
                     each_group<NC>([&](auto of) {
                         force(of);
                         collide(of);
                     });
                 } else {
                     each_group<NC>(force);
-                    ux = vmul(vfma(0.5f, Ftx, pk[0]), inv_rho);
-                    uy = vmul(vfma(0.5f, Fty, pk[1]), inv_rho);
+                    ux = vmul(vfma(0.5f, Ftx, jx), inv_rho);
+                    uy = vmul(vfma(0.5f, Fty, jy), inv_rho);
                     each_group<NC>(collide);
                 }
                 Fout[node] = Ftx;
                 Fout[nxy + node] = Fty;
             }
+            // grad rho~ of row y - 1, for its collision in the next iteration
+            each_group<NC>([&](auto of) {
+                using V = typename decltype(of)::V;
+                grad_rows<V>(of(rt[K]), of(rt[K2]), of(rs[K]), of(rs[K2]), of(rd[K]), of(rd[K1]), of(rd[K2]), stencil, of(gx),
+                             of(gy));
+            });
         }
         lf = lnew;
     };
@@ -401,14 +387,14 @@ __device__ __forceinline__ void march_chunk(const StepArgs& A, const Planes& P, 
 template <int NC, int ST, bool SPEC, bool NOALLOC, int MINB>
 __global__ void __launch_bounds__(32 * kMarchWarps, MINB)
     march_step(const __grid_constant__ StepArgs A, const __grid_constant__ Planes P, int strips, int chunk) {
-    extern __shared__ __align__(16) float4 smem_march[];
+    extern __shared__ __align__(16) float smem_march[];
     pdl_wait();
     const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
     const int w = blockIdx.x * kMarchWarps + warp;
     const int cy = w / strips, y0 = cy * chunk;
     if (y0 >= A.ny) return;
     const int x0 = (w - cy * strips) * kMarchCols;
-    march_chunk<NC, ST, SPEC, NOALLOC>(A, P, A.mixf, smem_march + warp * 3 * kSlotVecs<NC>, x0, y0, min(chunk, A.ny - y0));
+    march_chunk<NC, ST, SPEC, NOALLOC>(A, P, A.mixf, smem_march + warp * 3 * kParkWords<NC> * 32, x0, y0, min(chunk, A.ny - y0));
 }
 
 }  // namespace fmlbm
