@@ -126,9 +126,9 @@ template <int ST, int NC>
 cudaError_t launch_batch_reduce_nc(const fmlbm_batch* b) {
     batch_reduce<NC, ST><<<b->nwork, dim3(kTX, 8), 0, b->stream>>>(b->d_lat, b->d_work, b->nwork, b->d_prev,
                                                                    b->d_partial);
-    const int total = b->capacity * kBatchSums<NC>;
-    batch_reduce_final<NC><<<(total + 127) / 128, 128, 0, b->stream>>>(b->d_lat, b->capacity, b->d_partial,
-                                                                         b->d_out);
+    int used = b->capacity;  // slots above the last one stepping have no sums
+    while (used > 1 && !b->slots[used - 1].active) --used;
+    batch_reduce_final<NC><<<used * kBatchSums<NC>, kFinalThreads, 0, b->stream>>>(b->d_lat, b->d_partial, b->d_out);
     return cudaGetLastError();
 }
 template <int ST>

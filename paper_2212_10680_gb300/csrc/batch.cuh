@@ -127,16 +127,16 @@ __global__ void __launch_bounds__(kTX* 8) batch_reduce(BatchLattice* __restrict_
     if (tid < K) partial[(size_t)w * K + tid] = sums_strip<K, Real>(red, 0, tid, 0);
 }
 
+// One block per (lattice, sum), in the order of sum_columns (a thread per sum added a lattice's
+// items one after the other: 80 us of every check of a 16-lattice sweep).
 template <int NC>
-__global__ void batch_reduce_final(const BatchLattice* __restrict__ lat, int n, const double* __restrict__ partial,
-                                   double* __restrict__ out) {
+__global__ void __launch_bounds__(kFinalThreads) batch_reduce_final(const BatchLattice* __restrict__ lat,
+                                                                    const double* __restrict__ partial,
+                                                                    double* __restrict__ out) {
     constexpr int K = kBatchSums<NC>;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n * K) return;
-    const int l = k / K, q = k % K;
-    double v = 0.0;
-    for (int w = lat[l].item0; w < lat[l].item0 + lat[l].nitems; ++w) v += partial[(size_t)w * K + q];
-    out[k] = v;
+    const int l = blockIdx.x / K, q = blockIdx.x - l * K;
+    const double t = column_sum<K>(partial + (size_t)lat[l].item0 * K, lat[l].nitems, q);
+    if (threadIdx.x == 0) out[blockIdx.x] = t;
 }
 
 // The two phases of a lattice from its densities rho[N][ny][nx] (mass, double), read as
