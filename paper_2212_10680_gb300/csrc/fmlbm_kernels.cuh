@@ -138,6 +138,7 @@ struct StepArgs {
     void* diag_partial;
     void* rho_prev;  // [N][ny][nx] in the storage arithmetic type
     int have_prev;
+    void* rho_snap;  // marching step: receives the densities of the state it reads (null: none)
     void* fields;    // split step: scratch planes [split_planes][ny][nx] of the arithmetic type
     // rows [check_y0, check_y1) whose nodes the domain check covers (check_y1 = 0: all); a slab
     // of a decomposed lattice leaves out its ghost rows, whose update is discarded
@@ -1320,6 +1321,55 @@ __global__ void __launch_bounds__(kTX* kRedTY) reduce_partial(StepArgs A,
     const int tid = threadIdx.y * kTX + threadIdx.x;
     if (tid < NC + 2)
         partial[(size_t)(blockIdx.y * gridDim.x + blockIdx.x) * (NC + 2) + tid] = diag_strip<NC, Real>(red, 0, tid, 0);
+}
+
+// The same partial sums from a density field rho ([N][ny][nx]) and the snapshot prev, for steps
+// that write the densities of the state they read (the marching step).  Each thread takes two rows
+// as the lanes of packed float2 values: the same sums per row as one row per thread, at half the
+// instructions.  A block takes several strips and adds their rows up at the end, one lane per strip
+// and sum: a strip's 16 double additions cost the same for one lane as for 32 (one FP64 warp
+// instruction per 19 cycles and multiprocessor; the four sums of a strip by four warps instead of
+// four lanes cost 24 us more).  1024^2 binary: 13 us, bound by the latency of the sums' chain.
+constexpr int kRhoStrips = 4;                                // strips per block
+constexpr int kRhoGroups = 2;                                // strips at a time, four warps each
+template <int NC>
+__global__ void __launch_bounds__(kTX * 4 * kRhoGroups, 6) reduce_rho(const float* __restrict__ rho,
+                                                                  const float* __restrict__ prev, int nx, int ny,
+                                                                  int have_prev, int nstrips,
+                                                                  double* __restrict__ partial) {
+    constexpr int K = NC + 2, S = kRhoStrips;
+    pdl_wait();
+    __shared__ Sum2<float2> red[S][kRedTY / 2][K];
+    const int tiles_x = (nx + kTX - 1) / kTX, s0 = blockIdx.x * S;
+    const int ty = threadIdx.y & 3;
+    const size_t nxy = (size_t)nx * ny;
+    for (int j = threadIdx.y >> 2; j < S; j += kRhoGroups) {  // uniform over a warp
+        if (s0 + j >= nstrips) break;
+        const int row = (s0 + j) / tiles_x, col = s0 + j - row * tiles_x;
+        const int x = col * kTX + threadIdx.x, y = row * kRedTY + 2 * ty;
+        const size_t node = (size_t)y * nx + x;
+        const bool v0 = x < nx && y < ny, v1 = x < nx && y + 1 < ny;
+        float2 r[NC], pv[NC];
+#pragma unroll
+        for (int i = 0; i < NC; ++i) {
+            r[i] = make_float2(v0 ? rho[i * nxy + node] : 0.f, v1 ? rho[i * nxy + node + nx] : 0.f);
+            pv[i] = make_float2(v0 ? prev[i * nxy + node] : 0.f, v1 ? prev[i * nxy + node + nx] : 0.f);
+        }
+        Sum2<float2> acc[K];
+        diag_node<NC, float2>(r, pv, have_prev, acc);
+        diag_warp<NC, float2>(acc, red[j][ty]);
+    }
+    __syncthreads();
+    const int q = threadIdx.y * kTX + threadIdx.x, j = q / K, k = q - j * K;
+    if (j < S && s0 + j < nstrips) {
+        double v = 0.0;  // row by row, as sums_strip
+#pragma unroll
+        for (int w = 0; w < kRedTY; ++w) {
+            v += (double)lane(red[j][w / 2][k].hi, w & 1);
+            v += (double)lane(red[j][w / 2][k].lo, w & 1);
+        }
+        partial[(size_t)(s0 + j) * K + k] = v;
+    }
 }
 
 // Phase measure of a lattice: per component the sum over the nodes of ln rho_i, on the tiling

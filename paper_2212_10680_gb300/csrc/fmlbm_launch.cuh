@@ -135,6 +135,17 @@ inline cudaError_t launch_reduce_final(int nc, const void* partial, int nx, int 
     return cudaGetLastError();
 }
 
+// The partial sums of a state's diagnostics from its densities (reduce_rho; float storage, two or
+// three components), launched programmatically behind the step that writes them.
+inline cudaError_t launch_reduce_rho(int nc, const void* rho, const void* prev, int nx, int ny, int have_prev,
+                                     void* partial, cudaStream_t s) {
+    const int n = reduce_blocks(nx, ny);
+    const dim3 grid((n + kRhoStrips - 1) / kRhoStrips), block(kTX, 4 * kRhoGroups);
+    const float *r = static_cast<const float*>(rho), *p = static_cast<const float*>(prev);
+    return launch_kernel(nc == 2 ? reduce_rho<2> : reduce_rho<3>, grid, block, 0, s, true, r, p, nx, ny, have_prev, n,
+                         static_cast<double*>(partial));
+}
+
 // The specialised step (fused_step<..., SPEC = true>): float and 16-bit storage, 8-row tiles,
 // for lattices with the Peng-Robinson EOS, isotropic stencils, the lagged velocity reading and
 // the well-balanced formulation.
@@ -201,6 +212,13 @@ template <int NC, int ST, bool SPEC>
 cudaError_t launch_march(const StepArgs& A, cudaStream_t s) {
     return march_state_bytes<NC, ST>(A) <= kMarchL2Bytes ? launch_march_as<NC, ST, SPEC, true>(A, s)
                                                          : launch_march_as<NC, ST, SPEC, false>(A, s);
+}
+
+// Whether launch_step takes the marching step for these arguments (8-row tiles, no request).
+template <int ST>
+bool march_takes(const StepArgs& A, int nc) {
+    if (A.standard) return false;
+    return kSpecStep<ST> && (nc == 2 || nc == 3) && march_applies(A);
 }
 
 #define FMLBM_DEFINE_LAUNCHERS(ST)                                                                        \

@@ -199,6 +199,7 @@ __device__ __forceinline__ void march_chunk(const StepArgs& A, const Planes& P, 
     };
     const float* Fin = static_cast<const float*>(A.Fin);
     float* Fout = static_cast<float*>(A.Fout);
+    float* snap = static_cast<float*>(A.rho_snap);
     load_row();
     // rolling rows, indexed by the iteration mod 3: rho~ with its x-sums and x-differences, Phi
     // likewise (one row behind), ln f of the last row, grad rho~ of the row to collide next
@@ -225,6 +226,11 @@ __device__ __forceinline__ void march_chunk(const StepArgs& A, const Planes& P, 
                 }
                 const V r = sum9(h);
                 of(rt[K]) = vmul(r, of.of(m.invM));
+                if (snap != nullptr && it >= 2 && it < rows + 2 && own) {
+#pragma unroll
+                    for (int l = 0; l < (PAIR ? 2 : 1); ++l)
+                        snap[(size_t)(i0 + l) * nxy + (y0 + it - 2) * nx + xc] = fmlbm::lane(r, l);
+                }
             });
             park_put(slots + K * kParkWords<NC> * 32, lane, pk);
         }
