@@ -383,18 +383,18 @@ void fmlbm_destroy(fmlbm_handle* h);
 
 /* ------------------------------------------------------------------------------------
  * Batches: many independent lattices of one component count and storage precision
- * (any sizes, any mixtures) in slots, advanced together by one persistent kernel per
- * time step.  Each lattice's arithmetic is that of a single-lattice plain step, so its
+ * (any sizes, any mixtures) in slots, advanced together by one kernel per time step
+ * (two components in float or 16-bit storage on 8-row tiles: one per 48 lattices).  Each lattice's arithmetic is that of a single-lattice plain step, so its
  * results are bit-identical to fmlbm_step on its own handle, whatever else shares the
- * batch.  fmlbm_batch_run captures chunks of steps as a CUDA graph, checks every
- * lattice's residual after each chunk and retires it once converged.  Batches are not
+ * batch.  fmlbm_batch_run enqueues chunks of steps, checks every lattice's residual
+ * after each chunk and retires it once converged.  Batches are not
  * thread-safe.  The paper runs its envelope points as independent simulations
  * (Section V.B); a batch runs such sweeps side by side.
  * ------------------------------------------------------------------------------------ */
 typedef struct fmlbm_batch fmlbm_batch;
 
 /* capacity: maximum number of slots (1 .. 2^20).  cuda_stream: caller-owned stream, or
- * NULL for a stream the batch creates (graph capture needs a non-default stream). */
+ * NULL for a non-blocking stream that the batch creates. */
 fmlbm_status fmlbm_batch_create(int32_t n_components, int32_t precision, int32_t capacity, void* cuda_stream,
                                 fmlbm_batch** out);
 /* Adds a lattice in a free slot, initialised at rest from rho_host ([N][ny][nx] mass
@@ -414,7 +414,7 @@ fmlbm_status fmlbm_batch_step(fmlbm_batch* b, int64_t nsteps);
 fmlbm_status fmlbm_batch_check(fmlbm_batch* b);
 /* Runs every active slot until it retires: the batch's convergence measure (fmlbm_criterion:
  * the residual, or the phase-measure change, over the last check interval) < tol at a check
- * (every check_every steps, one graph launch per chunk), a latched error, or max_steps
+ * (every check_every steps), a latched error, or max_steps
  * reached (FMLBM_E_NOT_CONVERGED).  Outputs per slot (arrays of capacity entries, may be
  * NULL): steps taken, last value of the convergence measure, status. */
 fmlbm_status fmlbm_batch_run(fmlbm_batch* b, int64_t max_steps, int32_t check_every, double tol,
@@ -425,7 +425,7 @@ fmlbm_status fmlbm_batch_set_criterion(fmlbm_batch* b, int32_t criterion);
 /* Change of the phase measure of a slot over the last check interval (+inf before a second
  * check, NaN after a latched error); every check computes it beside the residual. */
 fmlbm_status fmlbm_batch_slot_phase_change(fmlbm_batch* b, int32_t slot, double* change);
-/* One graph-launched chunk of steps for every active slot followed by a check (the body
+/* One chunk of steps for every active slot followed by a check (the body
  * of fmlbm_batch_run without the retirement decisions; synchronises). */
 fmlbm_status fmlbm_batch_run_chunk(fmlbm_batch* b, int32_t steps);
 /* Steps taken, last residual (+inf before a second check), status and activity of a slot. */

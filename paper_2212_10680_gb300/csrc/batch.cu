@@ -1,7 +1,7 @@
 // Batched lattices (C ABI part of include/fmlbm.h): slots that hold independent
 // lattices of one component count and storage precision, advanced together by the
-// persistent batch kernel; graph-captured step chunks; per-lattice convergence checks
-// and retirement; a tile-shape / grid autotuner.
+// batch kernels; per-lattice convergence checks and retirement; a tile-shape / grid autotuner.
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -36,18 +36,21 @@ struct Slot {
     size_t bytes = 0;
 };
 
-template <int ST>
-cudaError_t launch_batch_step_st(int nc, int ty, BatchLattice* lat, const WorkItem* work, int nwork, int grid,
-                                 cudaStream_t s);
-
 }  // namespace
+
+// The parameters of one launch of the packed batch step.
+struct PackGroup {
+    int n = 0, blocks = 0;
+    int first[kBatchGroup] = {};
+    PackLattice lat[kBatchGroup];
+};
 
 struct fmlbm_batch {
     int nc = 0;
     int precision = 0;
     int capacity = 0;
     cudaStream_t stream = nullptr;
-    bool own_stream = false;    // created here (graph capture needs a non-default stream)
+    bool own_stream = false;    // created here
     int device = 0, sms = 1;
     std::vector<Slot> slots;
     BatchLattice* d_lat = nullptr;
@@ -57,6 +60,11 @@ struct fmlbm_batch {
     bool work_dirty = true;
     int tile_y = kTileYSmall;   // 8-row tiles, 4 blocks per SM: as the single-lattice step
     int grid_mult = 4;          // blocks = grid_mult * SMs (capped by the work count)
+    bool spec = false;          // every active lattice has the options of the specialised step
+    // launches of one packed step: [steps enqueued since they were made & 1]
+    std::vector<PackGroup> groups[2];
+    long long since = 0;
+    bool counted = false;       // a captured step's replays have their counts on the device only
     void** d_prev = nullptr;
     double* d_partial = nullptr;
     int partial_cap = 0;
@@ -65,8 +73,6 @@ struct fmlbm_batch {
     int criterion = FMLBM_CRITERION_RESIDUAL;
     ErrorLatch* d_err = nullptr;
     ErrorLatch* h_err = nullptr;  // pinned, capacity
-    cudaGraphExec_t graph = nullptr;
-    int graph_steps = 0;
     size_t bytes_in_use = 0;
     std::string last_error;
 };
@@ -85,40 +91,73 @@ fmlbm_status bfail(fmlbm_batch* b, fmlbm_status s, const std::string& m) {
 
 size_t rsize(int p) { return p == FMLBM_FP64 ? 8 : 4; }
 
+int grid_for(const fmlbm_batch* b) {
+    const int g = b->grid_mult * b->sms;
+    return b->nwork < g ? (b->nwork > 0 ? b->nwork : 1) : g;
+}
+
 template <int ST, int NC, int TY>
-cudaError_t launch_batch_step_t(BatchLattice* lat, const WorkItem* work, int nwork, int grid, cudaStream_t s) {
+cudaError_t launch_batch_step_t(const fmlbm_batch* b, int ahead, bool pdl) {
     using Real = typename StoreTraits<ST>::Real;
     constexpr size_t smem = sizeof(StepSmem<Real, NC, TY>);
     auto k = batch_step<NC, ST, TY>;
     FMLBM_ENSURE_SMEM(k, smem);
-    k<<<grid, dim3(kTX, TY), smem, s>>>(lat, work, nwork);
-    return cudaGetLastError();
+    return launch_kernel(k, dim3(grid_for(b)), dim3(kTX, TY), smem, b->stream, pdl, b->d_lat, (const WorkItem*)b->d_work,
+                         b->nwork, ahead);
+}
+template <int ST, bool SPEC, int MAXL>
+cudaError_t launch_batch_pack_as(const fmlbm_batch* b, const PackGroup& G, bool pdl) {
+    PackBatch<MAXL> B;
+    B.n = G.n;
+    std::memcpy(B.first, G.first, sizeof B.first);
+    std::memcpy(B.lat, G.lat, (size_t)G.n * sizeof(PackLattice));
+    constexpr size_t smem = sizeof(PackSmem<2, kTileYSmall>);
+    auto k = batch_pack<ST, SPEC, MAXL>;
+    FMLBM_ENSURE_SMEM(k, smem);
+    FMLBM_ENSURE_CARVEOUT(k, 35);  // as the packed step of a single lattice
+    return launch_kernel(k, dim3(G.blocks), dim3(kTX, kTileYSmall), smem, b->stream, pdl, B);
+}
+template <int ST, bool SPEC>
+cudaError_t launch_batch_pack(const fmlbm_batch* b, int ahead, bool pdl) {
+    for (const PackGroup& G : b->groups[(b->since + ahead) & 1]) {
+        const cudaError_t e = G.n <= kBatchGroupSmall ? launch_batch_pack_as<ST, SPEC, kBatchGroupSmall>(b, G, pdl)
+                                                      : launch_batch_pack_as<ST, SPEC, kBatchGroup>(b, G, pdl);
+        if (e != cudaSuccess) return e;
+        pdl = true;
+    }
+    return cudaSuccess;
 }
 
+// Two components in float or 16-bit storage: the packed step (1000 steps of 16 binaries of 88 to 484
+// nodes a side, FP32, with their creation and read-back: 62.8 ms by the persistent kernel, 46.5 packed).
+bool packed(const fmlbm_batch* b) { return b->nc == 2 && b->precision != FMLBM_FP64 && b->tile_y == kTileYSmall; }
+
 template <int ST, int NC>
-cudaError_t launch_batch_step_nc(int ty, BatchLattice* lat, const WorkItem* work, int nwork, int grid, cudaStream_t s) {
-    return ty == kTileYLarge ? launch_batch_step_t<ST, NC, kTileYLarge>(lat, work, nwork, grid, s)
-                             : launch_batch_step_t<ST, NC, kTileYSmall>(lat, work, nwork, grid, s);
+cudaError_t launch_batch_step_nc(const fmlbm_batch* b, int ahead, bool pdl) {
+    if (b->tile_y == kTileYLarge) return launch_batch_step_t<ST, NC, kTileYLarge>(b, ahead, pdl);
+    if constexpr (NC == 2 && kSpecStep<ST>) {
+        if (!b->counted) return b->spec ? launch_batch_pack<ST, true>(b, ahead, pdl) : launch_batch_pack<ST, false>(b, ahead, pdl);
+    }
+    return launch_batch_step_t<ST, NC, kTileYSmall>(b, ahead, pdl);
 }
 
 template <int ST>
-cudaError_t launch_batch_step_st(int nc, int ty, BatchLattice* lat, const WorkItem* work, int nwork, int grid,
-                                 cudaStream_t s) {
-    switch (nc) {
-        case 1: return launch_batch_step_nc<ST, 1>(ty, lat, work, nwork, grid, s);
-        case 2: return launch_batch_step_nc<ST, 2>(ty, lat, work, nwork, grid, s);
-        case 3: return launch_batch_step_nc<ST, 3>(ty, lat, work, nwork, grid, s);
-        case 4: return launch_batch_step_nc<ST, 4>(ty, lat, work, nwork, grid, s);
+cudaError_t launch_batch_step_st(const fmlbm_batch* b, int ahead, bool pdl) {
+    switch (b->nc) {
+        case 1: return launch_batch_step_nc<ST, 1>(b, ahead, pdl);
+        case 2: return launch_batch_step_nc<ST, 2>(b, ahead, pdl);
+        case 3: return launch_batch_step_nc<ST, 3>(b, ahead, pdl);
+        case 4: return launch_batch_step_nc<ST, 4>(b, ahead, pdl);
     }
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_batch_step(const fmlbm_batch* b, int ty, int grid) {
+cudaError_t launch_batch_step(const fmlbm_batch* b, int ahead, bool pdl) {
     switch (b->precision) {
-        case FMLBM_FP64: return launch_batch_step_st<ST_F64>(b->nc, ty, b->d_lat, b->d_work, b->nwork, grid, b->stream);
-        case FMLBM_FP32: return launch_batch_step_st<ST_F32>(b->nc, ty, b->d_lat, b->d_work, b->nwork, grid, b->stream);
-        case FMLBM_FP16DEV: return launch_batch_step_st<ST_F16DEV>(b->nc, ty, b->d_lat, b->d_work, b->nwork, grid, b->stream);
-        default: return launch_batch_step_st<ST_BF16DEV>(b->nc, ty, b->d_lat, b->d_work, b->nwork, grid, b->stream);
+        case FMLBM_FP64: return launch_batch_step_st<ST_F64>(b, ahead, pdl);
+        case FMLBM_FP32: return launch_batch_step_st<ST_F32>(b, ahead, pdl);
+        case FMLBM_FP16DEV: return launch_batch_step_st<ST_F16DEV>(b, ahead, pdl);
+        default: return launch_batch_step_st<ST_BF16DEV>(b, ahead, pdl);
     }
 }
 
@@ -148,17 +187,6 @@ cudaError_t launch_batch_reduce(const fmlbm_batch* b) {
         case FMLBM_FP16DEV: return launch_batch_reduce_st<ST_F16DEV>(b);
         default: return launch_batch_reduce_st<ST_BF16DEV>(b);
     }
-}
-
-int grid_for(const fmlbm_batch* b) {
-    const int g = b->grid_mult * b->sms;
-    return b->nwork < g ? (b->nwork > 0 ? b->nwork : 1) : g;
-}
-
-void drop_graph(fmlbm_batch* b) {
-    if (b->graph) cudaGraphExecDestroy(b->graph);
-    b->graph = nullptr;
-    b->graph_steps = 0;
 }
 
 // Descriptor of slot k (host side), both step parities.
@@ -192,22 +220,60 @@ void fill_descriptor(fmlbm_batch* b, int k) {
     d.tile_y = b->tile_y;
 }
 
+// The packed step's parameters of the active slots, for both parities.
+void fill_groups(fmlbm_batch* b) {
+    b->since = 0;
+    b->counted = false;
+    const bool dev16 = b->precision != FMLBM_FP32;
+    for (int p = 0; p < 2; ++p) {
+        std::vector<PackGroup>& gs = b->groups[p];
+        gs.clear();
+        if (!packed(b)) continue;
+        for (int k = 0; k < b->capacity; ++k) {
+            const Slot& s = b->slots[k];
+            if (!s.used || !s.active) continue;
+            if (gs.empty() || gs.back().n == kBatchGroup) gs.emplace_back();
+            const StepArgs& A = b->h_lat[k].args[(s.steps + p) & 1];
+            const Planes P = make_planes(A, 2, dev16, dev16 ? 2 : 4);
+            PackGroup& G = gs.back();
+            PackLattice& d = G.lat[G.n];
+            d.nx = A.nx;
+            d.ny = A.ny;
+            d.stencil = A.stencil;
+            d.lagged = A.lagged;
+            d.Fin = A.Fin;
+            d.Fout = A.Fout;
+            d.err = A.err;
+            std::copy(P.in, P.in + 18, d.in);
+            std::copy(P.out, P.out + 18, d.out);
+            std::copy(P.g0in, P.g0in + 2, d.g0in);
+            std::copy(P.g0out, P.g0out + 2, d.g0out);
+            d.mixf = A.mixf;
+            G.first[G.n++] = G.blocks;
+            G.blocks += b->h_lat[k].nitems;
+        }
+    }
+}
+
 // Rebuild the work list (active slots only, items of a slot contiguous) and upload the
 // descriptors.
 fmlbm_status rebuild(fmlbm_batch* b) {
     std::vector<WorkItem> items;
+    b->spec = true;
     for (int k = 0; k < b->capacity; ++k) {
         fill_descriptor(b, k);
         Slot& s = b->slots[k];
         BatchLattice& d = b->h_lat[k];
         d.item0 = (int)items.size();
         if (s.used && s.active) {
+            b->spec = b->spec && spec_options(d.args[0]);
             for (int y0 = 0; y0 < s.L.ny; y0 += b->tile_y)
                 for (int x0 = 0; x0 < s.L.nx; x0 += kTX) items.push_back(WorkItem{k, x0, y0});
         }
         d.nitems = (int)items.size() - d.item0;
     }
     b->nwork = (int)items.size();
+    fill_groups(b);
     if (b->nwork > b->work_cap) {
         if (b->d_work) cudaFree(b->d_work);
         if (b->d_partial) cudaFree(b->d_partial);
@@ -227,48 +293,29 @@ fmlbm_status rebuild(fmlbm_batch* b) {
     BCUDA(b, cudaMemcpyAsync(b->d_prev, prev.data(), prev.size() * sizeof(void*), cudaMemcpyHostToDevice, b->stream));
     BCUDA(b, cudaStreamSynchronize(b->stream));  // host vectors above are temporaries
     b->work_dirty = false;
-    drop_graph(b);
     return FMLBM_OK;
 }
 
 fmlbm_status ensure_work(fmlbm_batch* b) { return b->work_dirty ? rebuild(b) : FMLBM_OK; }
 
-// Enqueue n steps of all active slots (no synchronisation).
+// Enqueue n steps of all active slots (no synchronisation), launched programmatically behind one
+// another (serving 12 lattices of 64^2 to 184^2 took 26.0 ms with the launches of a check interval
+// captured in a graph, 24.0 ms with these).  Steps under stream capture, and those after them until
+// the next rebuild, choose their buffers by the counters on the device, which a replay advances.
 fmlbm_status enqueue_steps(fmlbm_batch* b, long long n) {
-    const int grid = grid_for(b);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    BCUDA(b, cudaStreamIsCapturing(b->stream, &cap));
+    const bool capturing = cap != cudaStreamCaptureStatusNone;
+    b->counted = b->counted || capturing;
     const int nb = (b->capacity + 127) / 128;
-    for (long long k = 0; k < n; ++k) {
-        BCUDA(b, launch_batch_step(b, b->tile_y, grid));
-        batch_advance<<<nb, 128, 0, b->stream>>>(b->d_lat, b->capacity);
+    for (long long done = 0; done < n;) {
+        const int m = (int)std::min<long long>(n - done, 1 << 20);
+        for (int k = 0; k < m; ++k) BCUDA(b, launch_batch_step(b, k, k > 0 && !capturing));
+        b->since += m;
+        batch_advance<<<nb, 128, 0, b->stream>>>(b->d_lat, b->capacity, m);
         BCUDA(b, cudaGetLastError());
+        done += m;
     }
-    for (auto& s : b->slots)
-        if (s.used && s.active) s.steps += n;
-    return FMLBM_OK;
-}
-
-// A chunk of n steps as one CUDA graph (captured once per membership and chunk length).
-fmlbm_status run_chunk(fmlbm_batch* b, int n) {
-    if (!b->graph || b->graph_steps != n) {
-        drop_graph(b);
-        cudaGraph_t g = nullptr;
-        BCUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-        std::vector<long long> saved;
-        for (auto& s : b->slots) saved.push_back(s.steps);
-        fmlbm_status st = enqueue_steps(b, n);
-        for (size_t k = 0; k < saved.size(); ++k) b->slots[k].steps = saved[k];
-        cudaError_t e = cudaStreamEndCapture(b->stream, &g);
-        if (st != FMLBM_OK) {
-            if (g) cudaGraphDestroy(g);
-            return st;
-        }
-        if (e != cudaSuccess) return bfail(b, FMLBM_E_CUDA, std::string("capture: ") + cudaGetErrorString(e));
-        e = cudaGraphInstantiate(&b->graph, g, 0);
-        cudaGraphDestroy(g);
-        if (e != cudaSuccess) return bfail(b, FMLBM_E_CUDA, std::string("instantiate: ") + cudaGetErrorString(e));
-        b->graph_steps = n;
-    }
-    BCUDA(b, cudaGraphLaunch(b->graph, b->stream));
     for (auto& s : b->slots)
         if (s.used && s.active) s.steps += n;
     return FMLBM_OK;
@@ -395,7 +442,6 @@ fmlbm_status fmlbm_batch_create(int32_t n_components, int32_t precision, int32_t
 void fmlbm_batch_destroy(fmlbm_batch* b) {
     if (!b) return;
     cudaStreamSynchronize(b->stream);
-    drop_graph(b);
     for (auto& s : b->slots)
         if (s.used) free_slot(b, s);
     cudaStreamSynchronize(b->stream);
@@ -533,7 +579,7 @@ fmlbm_status fmlbm_batch_run(fmlbm_batch* b, int64_t max_steps, int32_t check_ev
         const int n = (int)std::min<long long>(check_every, std::max<long long>(left, 1));
         st = ensure_work(b);
         if (st != FMLBM_OK) return st;
-        st = run_chunk(b, n);
+        st = enqueue_steps(b, n);
         if (st != FMLBM_OK) return st;
         st = check_all(b);
         if (st != FMLBM_OK) return st;
@@ -565,7 +611,7 @@ fmlbm_status fmlbm_batch_run_chunk(fmlbm_batch* b, int32_t steps) {
     if (!b || steps < 1) return bfail(b, FMLBM_E_INVALID_ARG, "bad argument");
     fmlbm_status st = ensure_work(b);
     if (st != FMLBM_OK || b->nwork == 0) return st;
-    st = run_chunk(b, steps);
+    st = enqueue_steps(b, steps);
     if (st != FMLBM_OK) return st;
     return check_all(b);
 }

@@ -1,22 +1,22 @@
 // Batched lattices: many independent lattices (same component count and storage,
-// any sizes, any mixtures) advanced together by one persistent kernel per time step.
+// any sizes, any mixtures) advanced together by one kernel per time step.
 //
 // Every lattice has a device-resident descriptor holding its StepArgs for both
 // step parities (the ping-pong buffers swapped) and its own step counter.  A work list
 // of (lattice, tile) items covers all lattices; a block copies the descriptor of its
 // item's lattice into shared memory and runs the same phase functions as fused_step,
 // so each lattice's arithmetic is exactly that of a single-lattice plain step: results
-// are bit-identical alone and in any mix.  Retired lattices are skipped through a
-// device flag, so a captured graph of the step loop stays valid as lattices retire.
+// are bit-identical alone and in any mix.  Two components in float or 16-bit storage take the
+// packed step's tiles, with the descriptors in the launch's parameters (batch_pack).
 #pragma once
 
-#include "fmlbm_kernels.cuh"
+#include "fmlbm_pack.cuh"
 
 namespace fmlbm {
 
 struct BatchLattice {
     StepArgs args[2];    // [step & 1]
-    long long step;      // steps taken (device side, advanced by batch_advance)
+    long long step;      // steps taken before the launches in flight (advanced by batch_advance)
     int active;          // 0: retired or not started
     int item0, nitems;   // its items in the work list
     int tile_y;          // the tile height its items were cut with
@@ -28,12 +28,13 @@ struct WorkItem {
     int x0, y0;
 };
 
-// One step of every active lattice.
+// One step of every active lattice, `ahead` steps after the counters.
 // Float storage capped at 64 registers (1024 threads per SM), as the single-lattice step.
 template <int NC, int ST, int TY>
 __global__ void __launch_bounds__(kTX* TY, ST == ST_F64 ? 1 : 1024 / (kTX * TY)) batch_step(BatchLattice* __restrict__ lat,
-                                                      const WorkItem* __restrict__ work, int nwork) {
+                                                      const WorkItem* __restrict__ work, int nwork, int ahead) {
     using Real = typename StoreTraits<ST>::Real;
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_batch[];
     auto& S = *reinterpret_cast<StepSmem<Real, NC, TY>*>(smem_batch);
     __shared__ __align__(16) StepArgs As;
@@ -46,7 +47,7 @@ __global__ void __launch_bounds__(kTX* TY, ST == ST_F64 ? 1 : 1024 / (kTX * TY))
         const WorkItem it = work[w];
         const BatchLattice* L = lat + it.lattice;
         if (!L->active) continue;  // uniform across the block
-        const int* src = reinterpret_cast<const int*>(&L->args[L->step & 1]);
+        const int* src = reinterpret_cast<const int*>(&L->args[(L->step + ahead) & 1]);
         int* dst = reinterpret_cast<int*>(&As);
         for (int k = tid; k < WORDS; k += NT) dst[k] = src[k];
         __syncthreads();
@@ -67,9 +68,53 @@ __global__ void __launch_bounds__(kTX* TY, ST == ST_F64 ? 1 : 1024 / (kTX * TY))
     }
 }
 
-__global__ void batch_advance(BatchLattice* __restrict__ lat, int n) {
+// One step of up to MAXL lattices of two components in float or 16-bit storage on 8-row tiles: the
+// packed step's tiles, one block each, with the lattices' descriptors in the launch's parameters.
+// A block finds its lattice by its index (the descriptors are in the order of their tiles) in
+// registers that the whole warp shares, and reads plane addresses and mixture constants as
+// constants, so that a block starts with its loads.  A step of 16 binaries of 88 to 484 nodes a side
+// (971,000 nodes, FP32) takes 38.0 us, one of 12 of 64^2 to 184^2 9.8; with the descriptor copied from
+// global to shared memory by every block 49.2 and 12.3 (two dependent reads and a barrier before
+// the first load, and a shared-memory read for each address), with four blocks per multiprocessor
+// 41.8 and 10.2.
+struct PackLattice {
+    int nx, ny, stencil, lagged;
+    const void* Fin;
+    void* Fout;
+    ErrorLatch* err;
+    const void* in[2 * 9];  // as Planes
+    void* out[2 * 9];
+    const float* g0in[2];
+    float* g0out[2];
+    MixConstT<float> mixf;
+};
+__device__ __forceinline__ bool checked_row(const PackLattice&, int) { return true; }
+constexpr int kBatchGroup = 48;       // lattices in one launch (27 KB of parameters)
+constexpr int kBatchGroupSmall = 16;  // fewer lattices take the launch with less to copy
+template <int MAXL>
+struct PackBatch {
+    int n;
+    int first[kBatchGroup];  // first block of each lattice
+    PackLattice lat[MAXL];
+};
+template <int ST, bool SPEC, int MAXL>
+__global__ void __launch_bounds__(kTX * 8, 5) batch_pack(const __grid_constant__ PackBatch<MAXL> B) {
+    pdl_wait();
+    extern __shared__ __align__(16) unsigned char smem_batch_pack[];
+    int l = 0;
+#pragma unroll
+    for (int s = MAXL > 32 ? 32 : MAXL / 2; s > 0; s >>= 1)
+        if (l + s < B.n && B.first[l + s] <= (int)blockIdx.x) l += s;
+    const PackLattice& L = B.lat[l];
+    const int t = blockIdx.x - B.first[l], cols = (L.nx + kTX - 1) / kTX, row = t / cols;
+    pack_tile<2, ST, SPEC, false>(L, L, *reinterpret_cast<PackSmem<2, 8>*>(smem_batch_pack), nullptr,
+                                  (t - row * cols) * kTX, row * 8, 0, 0, 0);
+}
+
+// Counts n steps on every active lattice.
+__global__ void batch_advance(BatchLattice* __restrict__ lat, int nlat, int n) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n && lat[k].active) lat[k].step += 1;
+    if (k < nlat && lat[k].active) lat[k].step += n;
 }
 
 // Per-item partial sums (2 NC + 2 doubles: sum rho_i, sum (rho - rho_prev)^2, sum rho^2, then

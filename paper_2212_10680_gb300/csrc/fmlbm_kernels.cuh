@@ -241,8 +241,8 @@ template <bool CG, typename E> __device__ __forceinline__ E ldsel(const E* p) {
 // index: each access address is then a single multiply-add onto a parameter, where the
 // forms above compute a 64-bit plane offset (two-component step: +1.5% on GB300; with
 // three components it cost registers and spilled).  CG: L2-only loads (ldcg).
-template <int ST, bool CG = false>
-__device__ __forceinline__ typename StoreTraits<ST>::Real load_gp(const Planes& P, int i, int a, int node) {
+template <int ST, bool CG = false, typename PL = Planes>
+__device__ __forceinline__ typename StoreTraits<ST>::Real load_gp(const PL& P, int i, int a, int node) {
     using Elem = typename StoreTraits<ST>::Elem;
     if constexpr (ST == ST_F64 || ST == ST_F32) {
         return to_real(ldsel<CG>(static_cast<const Elem*>(P.in[i * 9 + a]) + node));
@@ -251,8 +251,8 @@ __device__ __forceinline__ typename StoreTraits<ST>::Real load_gp(const Planes& 
         return to_real(ldsel<CG>(static_cast<const Elem*>(P.in[i * 8 + a - 1]) + node));
     }
 }
-template <int ST>
-__device__ __forceinline__ void store_gp(const Planes& P, int i, int a, int node, typename StoreTraits<ST>::Real v) {
+template <int ST, typename PL = Planes>
+__device__ __forceinline__ void store_gp(const PL& P, int i, int a, int node, typename StoreTraits<ST>::Real v) {
     using Elem = typename StoreTraits<ST>::Elem;
     if constexpr (ST == ST_F64 || ST == ST_F32) {
         static_cast<Elem*>(P.out[i * 9 + a])[node] = v;
@@ -601,8 +601,8 @@ __device__ __forceinline__ void pull_rho(const StepArgs& A, int wx, int wy, bool
 
 // Latch the first node that left the EOS domain (rho~_i <= 0, beta >= 1, non-finite ln f).
 // Lane k is the node (x + k dx, y); valid_mask bit k says whether it lies in the lattice.
-template <int NC, typename V>
-__device__ __forceinline__ void domain_check(const StepArgs& A, const V* rt, const V* lnf, V beta, int x, int dx,
+template <int NC, typename V, typename AT = StepArgs>
+__device__ __forceinline__ void domain_check(const AT& A, const V* rt, const V* lnf, V beta, int x, int dx,
                                              int y, unsigned valid_mask) {
     using E = LaneE<V>;
 #pragma unroll

@@ -75,8 +75,8 @@ __device__ __forceinline__ void pack_phi(const MixConstT<float>& m, PackSmem<NC,
 }
 
 // The pulled values of a node: the nine of component i through the plane base addresses.
-template <int NC, int ST>
-__device__ __forceinline__ void pack_pull(const Planes& P, bool inner, int wx, int wy, int nx, int ny, Comps<NC> (&g)[9]) {
+template <int NC, int ST, typename PL>
+__device__ __forceinline__ void pack_pull(const PL& P, bool inner, int wx, int wy, int nx, int ny, Comps<NC> (&g)[9]) {
     const int node = wy * nx + wx;
     int xm = wx - 1, xp = wx + 1, ym = wy - 1, yp = wy + 1;
     if (!inner) {
@@ -106,24 +106,22 @@ __device__ __forceinline__ void pack_rho(const MixConstT<float>& m, const Comps<
     });
 }
 
+// One tile of the packed step: of a lattice's StepArgs and Planes, or of a batch's descriptor with
+// the members used here.  DIAG: the sums of a diagnostics request where A asks for them, with pv_s
+// their shared memory and the tile's place (row, col of cols) in their order.
 // SPEC: the Peng-Robinson EOS, isotropic stencils and the lagged velocity as constants.
-template <int NC, int ST, bool SPEC, int MINB>
-__global__ void __launch_bounds__(kTX * 8, MINB) pack_step(const __grid_constant__ StepArgs A,
-                                                          const __grid_constant__ Planes P) {
+template <int NC, int ST, bool SPEC, bool DIAG, typename AT, typename PL>
+__device__ __forceinline__ void pack_tile(const AT& A, const PL& P, PackSmem<NC, 8>& S, float* pv_s, int x0, int y0,
+                                          int row, int col, int cols) {
     constexpr int TY = 8, NT = kTX * TY;
-    pdl_wait();
-    extern __shared__ __align__(16) unsigned char smem_pack[];
-    auto& S = *reinterpret_cast<PackSmem<NC, TY>*>(smem_pack);
-    float* pv_s = reinterpret_cast<float*>(smem_pack + sizeof(PackSmem<NC, TY>));
     const MixConstT<float>& m = A.mixf;
     const int nx = A.nx, ny = A.ny, nxy = nx * ny;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kTX + tx;
-    const int x0 = blockIdx.x * kTX, y0 = blockIdx.y * TY;
     const int x = x0 + tx, y = y0 + ty;
     const bool valid = x < nx && y < ny;
     const int eos = SPEC ? 0 : -1, stencil = SPEC ? 0 : A.stencil;
     const bool lagged = SPEC ? true : A.lagged != 0;
-    diag_prefetch<NC, float, TY>(A, pv_s, tx, ty, x, y);
+    if constexpr (DIAG) diag_prefetch<NC, float, TY>(A, pv_s, tx, ty, x, y);
     if (lagged && valid) {
         const float* Fin = static_cast<const float*>(A.Fin);
         const int node = y * nx + x;
@@ -273,12 +271,23 @@ __global__ void __launch_bounds__(kTX * 8, MINB) pack_step(const __grid_constant
         Fout[node] = Ftx;
         Fout[(size_t)nxy + node] = Fty;
     }
-    if (A.diag_partial != nullptr) {  // uniform: diagnostics of the state this step read
-        float rr[NC];
+    if constexpr (DIAG) {
+        if (A.diag_partial != nullptr) {  // uniform: diagnostics of the state this step read
+            float rr[NC];
 #pragma unroll
-        for (int i = 0; i < NC; ++i) rr[i] = comp(r, i);
-        diag_tile<NC, float, TY>(A, rr, pv_s, tx, ty, x, y, y0, blockIdx.y, blockIdx.x, gridDim.x);
+            for (int i = 0; i < NC; ++i) rr[i] = comp(r, i);
+            diag_tile<NC, float, TY>(A, rr, pv_s, tx, ty, x, y, y0, row, col, cols);
+        }
     }
+}
+template <int NC, int ST, bool SPEC, int MINB>
+__global__ void __launch_bounds__(kTX * 8, MINB) pack_step(const __grid_constant__ StepArgs A,
+                                                          const __grid_constant__ Planes P) {
+    pdl_wait();
+    extern __shared__ __align__(16) unsigned char smem_pack[];
+    pack_tile<NC, ST, SPEC, true>(A, P, *reinterpret_cast<PackSmem<NC, 8>*>(smem_pack),
+                                  reinterpret_cast<float*>(smem_pack + sizeof(PackSmem<NC, 8>)), blockIdx.x * kTX,
+                                  blockIdx.y * 8, blockIdx.y, blockIdx.x, gridDim.x);
 }
 template <int NC>
 constexpr size_t pack_smem_bytes() {

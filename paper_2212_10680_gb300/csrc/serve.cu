@@ -3,7 +3,7 @@
 // A worker thread owns the batch and its stream.  Between chunks of steps it admits
 // queued requests in arrival order while a slot is free and the requests' device
 // bytes fit the budget (head-of-line: a request that does not fit waits for memory to
-// free up, later ones wait behind it), runs one graph-captured chunk for every
+// free up, later ones wait behind it), runs one chunk of steps for every
 // admitted lattice, checks residuals and phase measures, and retires each lattice at its own
 // criterion (the configured measure below tol, a latched error, or its step limit), copying its final
 // densities out and freeing its memory.  Each lattice's arithmetic is unaffected by
