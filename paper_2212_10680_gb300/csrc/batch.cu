@@ -357,6 +357,16 @@ fmlbm_status check_all(fmlbm_batch* b) {
     return FMLBM_OK;
 }
 
+template <int NC>
+cudaError_t launch_phase_nodes(const double* rho, int nx, int ny, const MixConst& m, PhaseNodes* part, double* out,
+                               cudaStream_t s) {
+    const long long nblk = (long long)((nx + 1) / 2) * ((ny + 1) / 2);
+    const int blocks = (int)std::min<long long>((nblk + kPhaseThreads - 1) / kPhaseThreads, kPhaseBlocks);
+    phase_nodes<NC><<<blocks, kPhaseThreads, 0, s>>>(rho, nx, ny, m, part);
+    phase_pick<NC><<<1, kPhaseThreads, 0, s>>>(rho, nx, ny, m, part, blocks, out);
+    return cudaGetLastError();
+}
+
 // The value fmlbm_batch_run compares with tol: the residual or the phase-measure change.
 double slot_measure(const fmlbm_batch* b, const Slot& s) {
     return b->criterion == FMLBM_CRITERION_PHASE ? s.phase_change : s.residual;
@@ -671,18 +681,19 @@ fmlbm_status fmlbm_batch_phases(fmlbm_batch* b, int32_t slot, double* rho_liquid
     Slot& s = b->slots[slot];
     const size_t nxy = (size_t)s.L.nx * s.L.ny;
     double* d = nullptr;
-    BCUDA(b, cudaMallocAsync((void**)&d, ((size_t)b->nc * nxy + 2 * kMaxC) * sizeof(double), b->stream));
+    const size_t rb = (size_t)b->nc * nxy * sizeof(double);
+    BCUDA(b, cudaMallocAsync((void**)&d, rb + 2 * kMaxC * sizeof(double) + kPhaseBlocks * sizeof(PhaseNodes), b->stream));
     double* out = d + (size_t)b->nc * nxy;
+    PhaseNodes* part = reinterpret_cast<PhaseNodes*>(out + 2 * kMaxC);
     cudaError_t e = launch_slot_moments(b, slot, d, nullptr, nullptr);
     if (e == cudaSuccess) {
         const MixConst& m = b->h_lat[slot].args[0].mixd;
         switch (b->nc) {
-            case 1: phase_nodes<1><<<1, kPhaseThreads, 0, b->stream>>>(d, s.L.nx, s.L.ny, m, out); break;
-            case 2: phase_nodes<2><<<1, kPhaseThreads, 0, b->stream>>>(d, s.L.nx, s.L.ny, m, out); break;
-            case 3: phase_nodes<3><<<1, kPhaseThreads, 0, b->stream>>>(d, s.L.nx, s.L.ny, m, out); break;
-            default: phase_nodes<4><<<1, kPhaseThreads, 0, b->stream>>>(d, s.L.nx, s.L.ny, m, out); break;
+            case 1: e = launch_phase_nodes<1>(d, s.L.nx, s.L.ny, m, part, out, b->stream); break;
+            case 2: e = launch_phase_nodes<2>(d, s.L.nx, s.L.ny, m, part, out, b->stream); break;
+            case 3: e = launch_phase_nodes<3>(d, s.L.nx, s.L.ny, m, part, out, b->stream); break;
+            default: e = launch_phase_nodes<4>(d, s.L.nx, s.L.ny, m, part, out, b->stream); break;
         }
-        e = cudaGetLastError();
     }
     double h[2 * kMaxC];
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, out, 2 * b->nc * sizeof(double), cudaMemcpyDeviceToHost, b->stream);

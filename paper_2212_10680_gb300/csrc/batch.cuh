@@ -194,9 +194,15 @@ __global__ void __launch_bounds__(kFinalThreads) batch_reduce_final(const BatchL
 // sublattice is then out of equilibrium on its own; the block mean is the thermodynamic state.
 // out = the block-mean molar densities rho~_i at the block of largest total molar density
 // sum_i rho_i / M_i (liquid) [N], then at the block of smallest (vapour) [N]; ties to the
-// lowest block index (row-major).  One block of threads, grid-stride over the node blocks, a
-// fixed-order tree: deterministic.
+// lowest block index (row-major): a choice, so the same however the node blocks are divided among
+// thread blocks.  Bound by its double divisions (N for each node), hence many thread blocks: with one
+// 350 us on average over 16 lattices of 8,600 to 171,000 nodes.
 constexpr int kPhaseThreads = 512;
+constexpr int kPhaseBlocks = 256;
+struct PhaseNodes {      // the largest and smallest density seen and their node blocks (-1: none)
+    double hi, lo;
+    long long ih, il;
+};
 __device__ __forceinline__ void block_nodes(long long k, int nx, int ny, long long (&node)[4]) {
     const int bxn = (nx + 1) / 2;
     const int x0 = 2 * (int)(k % bxn), y0 = 2 * (int)(k / bxn);
@@ -207,17 +213,38 @@ __device__ __forceinline__ void block_nodes(long long k, int nx, int ny, long lo
     node[3] = (long long)y1 * nx + x1;
 }
 
+// The block's choice from every thread's, in thread 0's result.
+__device__ __forceinline__ PhaseNodes phase_reduce(const PhaseNodes& mine) {
+    __shared__ PhaseNodes v[kPhaseThreads];
+    const int t = threadIdx.x;
+    v[t] = mine;
+    __syncthreads();
+    for (int w = kPhaseThreads / 2; w > 0; w >>= 1) {
+        if (t < w) {
+            const PhaseNodes o = v[t + w];
+            if (o.ih >= 0 && (v[t].ih < 0 || o.hi > v[t].hi || (o.hi == v[t].hi && o.ih < v[t].ih))) {
+                v[t].hi = o.hi;
+                v[t].ih = o.ih;
+            }
+            if (o.il >= 0 && (v[t].il < 0 || o.lo < v[t].lo || (o.lo == v[t].lo && o.il < v[t].il))) {
+                v[t].lo = o.lo;
+                v[t].il = o.il;
+            }
+        }
+        __syncthreads();
+    }
+    return v[0];
+}
+
 template <int NC>
 __global__ void __launch_bounds__(kPhaseThreads) phase_nodes(const double* __restrict__ rho, int nx, int ny,
-                                                             MixConstT<double> m, double* __restrict__ out) {
-    __shared__ double vmax[kPhaseThreads], vmin[kPhaseThreads];
-    __shared__ long long imax[kPhaseThreads], imin[kPhaseThreads];
+                                                             MixConstT<double> m, PhaseNodes* __restrict__ part) {
     const long long nxy = (long long)nx * ny;
     const long long nblk = (long long)((nx + 1) / 2) * ((ny + 1) / 2);
-    const int t = threadIdx.x;
     double hi = -1.0, lo = 0.0;
     long long ih = -1, il = -1;
-    for (long long k = t; k < nblk; k += kPhaseThreads) {
+    for (long long k = (long long)blockIdx.x * kPhaseThreads + threadIdx.x; k < nblk;
+         k += (long long)gridDim.x * kPhaseThreads) {
         long long node[4];
         block_nodes(k, nx, ny, node);
         double s = 0.0;
@@ -228,24 +255,22 @@ __global__ void __launch_bounds__(kPhaseThreads) phase_nodes(const double* __res
         if (ih < 0 || s > hi) { hi = s; ih = k; }          // k increases: first maximum kept
         if (il < 0 || s < lo) { lo = s; il = k; }
     }
-    vmax[t] = hi; imax[t] = ih; vmin[t] = lo; imin[t] = il;
-    __syncthreads();
-    for (int w = kPhaseThreads / 2; w > 0; w >>= 1) {
-        if (t < w) {
-            const int o = t + w;
-            if (imax[o] >= 0 && (imax[t] < 0 || vmax[o] > vmax[t] || (vmax[o] == vmax[t] && imax[o] < imax[t]))) {
-                vmax[t] = vmax[o]; imax[t] = imax[o];
-            }
-            if (imin[o] >= 0 && (imin[t] < 0 || vmin[o] < vmin[t] || (vmin[o] == vmin[t] && imin[o] < imin[t]))) {
-                vmin[t] = vmin[o]; imin[t] = imin[o];
-            }
-        }
-        __syncthreads();
-    }
+    const PhaseNodes best = phase_reduce(PhaseNodes{hi, lo, ih, il});
+    if (threadIdx.x == 0) part[blockIdx.x] = best;
+}
+
+template <int NC>
+__global__ void __launch_bounds__(kPhaseThreads) phase_pick(const double* __restrict__ rho, int nx, int ny,
+                                                            MixConstT<double> m, const PhaseNodes* __restrict__ part,
+                                                            int nparts, double* __restrict__ out) {
+    static_assert(kPhaseBlocks <= kPhaseThreads, "one thread per partial choice");
+    const int t = threadIdx.x;
+    const PhaseNodes best = phase_reduce(t < nparts ? part[t] : PhaseNodes{-1.0, 0.0, -1, -1});
+    const long long nxy = (long long)nx * ny;
     if (t < 2 * NC) {
         const int i = t % NC;
         long long node[4];
-        block_nodes(t < NC ? imax[0] : imin[0], nx, ny, node);
+        block_nodes(t < NC ? best.ih : best.il, nx, ny, node);
         double v = 0.0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) v += rho[i * nxy + node[q]] / m.M[i];
