@@ -51,6 +51,7 @@ struct fmlbm_handle {
     cudaStream_t tail = nullptr;     // final sums and copies of fused requests (non-blocking)
     cudaEvent_t part_ev[kDiagSlots] = {};    // [ticket % kDiagSlots]: partial sums of a fused request written
     cudaEvent_t tail_done[kDiagSlots] = {};  // [ticket % kDiagSlots]: the tail that read them has finished
+    bool tail_open[kDiagSlots] = {};         // and no host call has waited for its end yet
     double* diag_host = nullptr;     // pinned: kDiagSlots x kDiagWords doubles (results + error latch)
     cudaEvent_t diag_ev[kDiagSlots] = {};
     DiagSlot slot[kDiagSlots];
@@ -372,20 +373,6 @@ cudaError_t dispatch_reduce(fmlbm_handle* h, const StepArgs& A, void* partial, d
     }
 }
 
-// Calls that a stream capture in global mode elsewhere forbids to every thread (an event query, an
-// allocation), made for streams that are not being captured.
-struct RelaxedCapture {
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
-    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
-};
-bool event_done(cudaEvent_t e) {
-    RelaxedCapture relaxed;
-    if (cudaEventQuery(e) == cudaSuccess) return true;
-    cudaGetLastError();
-    return false;
-}
-
 // Whether a pending request is served by a marching step that writes the densities of the state it
 // reads and a reduction over them (every step of a 1024^2 binary asked: 46.5 us per step, with the
 // sums fused into tile steps 48.5).  Not under capture: the two snapshots swap with every request.
@@ -399,11 +386,15 @@ bool serve_by_snapshot(fmlbm_handle* h, const StepArgs& A, bool capturing) {
         case FMLBM_BF16DEV: takes = march_takes<ST_BF16DEV>(A, h->nc); break;
         default: break;
     }
-    RelaxedCapture relaxed;
-    if (takes && !h->rho_next &&
-        cudaMalloc(&h->rho_next, (size_t)h->nc * h->lattice.nx * h->lattice.ny * sizeof(float)) != cudaSuccess) {
-        cudaGetLastError();
-        h->rho_next = nullptr;
+    if (takes && !h->rho_next) {
+        // a stream capture in global mode elsewhere forbids every thread to allocate
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (cudaMalloc(&h->rho_next, (size_t)h->nc * h->lattice.nx * h->lattice.ny * sizeof(float)) != cudaSuccess) {
+            cudaGetLastError();
+            h->rho_next = nullptr;
+        }
+        cudaThreadExchangeStreamCaptureMode(&mode);
     }
     return takes && h->rho_next;
 }
@@ -485,6 +476,7 @@ double* result_slot(const fmlbm_handle* h, int64_t ticket) { return h->diag_dev 
 // on stream s), copy of the results and of the error latch into its host slot, event.
 fmlbm_status enqueue_diag_tail(fmlbm_handle* h, int64_t ticket, cudaStream_t s, bool final_sum, bool capturing) {
     DiagSlot& sl = h->slot[ticket % kDiagSlots];
+    h->tail_open[ticket % kDiagSlots] = true;
     double* host = h->diag_host + (size_t)(ticket % kDiagSlots) * kDiagWords;
     // the final sum writes the sums and, after them, the error latch into the result slot
     // (the standalone reduction did the same), so one copy brings both to the host
@@ -837,7 +829,7 @@ fmlbm_status fmlbm_step(fmlbm_handle* h, int64_t nsteps) {
         A.pdl = A.pdl_chain = pdl;
         if (fused >= 0) {  // this step also reduces the state it reads
             // the tail of request fused - kDiagSlots may still read this set of partial sums
-            if (!capturing && !event_done(h->tail_done[fused % kDiagSlots])) {
+            if (!capturing && h->tail_open[fused % kDiagSlots]) {
                 FM_CUDA(h, cudaStreamWaitEvent(h->stream, h->tail_done[fused % kDiagSlots], 0));
                 A.pdl = 0;
             }
@@ -1088,6 +1080,7 @@ fmlbm_status fmlbm_diagnostics_wait(fmlbm_handle* h, int64_t ticket, double* mas
         if (s != FMLBM_OK) return s;
     }
     FM_CUDA(h, cudaEventSynchronize(h->diag_ev[ticket % kDiagSlots]));
+    h->tail_open[ticket % kDiagSlots] = false;
     const double* d = h->diag_host + (size_t)(ticket % kDiagSlots) * kDiagWords;
     ErrorLatch latch;
     std::memcpy(&latch, d + kMaxC + 2, sizeof latch);
