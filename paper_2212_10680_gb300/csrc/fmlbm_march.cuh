@@ -50,7 +50,12 @@ template <int NC, int ST>
 inline size_t march_state_bytes(const StepArgs& A) {  // distributions and stored force a step reads
     return (size_t)A.nx * A.ny * (ST == ST_F32 ? NC * 36 + 8 : NC * 20 + 8);
 }
-inline bool march_applies(const StepArgs& A) { return (size_t)A.nx * A.ny >= kMarchNodes; }
+// Nor where the last strip is mostly empty: 64 columns take three strips (64 x 9000 ternary FP16 29.0 ->
+// 29.9 us, binary FP32 22.8 -> 22.4); a quarter more columns than the lattice has is the limit.
+inline bool march_applies(const StepArgs& A) {
+    const long long cols = (A.nx + kMarchCols - 1) / kMarchCols * kMarchCols;
+    return (size_t)A.nx * A.ny >= kMarchNodes && 4 * cols <= 5LL * A.nx;
+}
 // Rows per chunk: all warps resident at once (one wave of `capacity` warps) while that keeps a
 // chunk below 96 rows; otherwise as many waves as bring it there (4096^2 BF16 binary, 256 rows in
 // one wave 529 us, 125 rows in two 416 us).
