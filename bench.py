@@ -37,7 +37,10 @@ ALGO_BYTES = {"fp64": 144.0, "fp32": 72.0, "fp16dev": 40.0, "bf16dev": 40.0, "fp
 L2_FLUSH_BYTES = 256 << 20
 KERNEL_SOURCES = ["paper_2212_10680_gb300/csrc/fmlbm_lanes.cuh", "paper_2212_10680_gb300/csrc/fmlbm_kernels.cuh",
                   "paper_2212_10680_gb300/csrc/fmlbm_pair.cuh", "paper_2212_10680_gb300/csrc/fmlbm_launch.cuh",
-                  "paper_2212_10680_gb300/csrc/fmlbm_tma.cuh", "paper_2212_10680_gb300/csrc/fmlbm_multi.cuh"]
+                  "paper_2212_10680_gb300/csrc/fmlbm_tma.cuh", "paper_2212_10680_gb300/csrc/fmlbm_multi.cuh",
+                  "paper_2212_10680_gb300/csrc/fmlbm_comps.cuh", "paper_2212_10680_gb300/csrc/fmlbm_march.cuh",
+                  "paper_2212_10680_gb300/csrc/fmlbm_pack.cuh", "paper_2212_10680_gb300/csrc/fmlbm_split.cuh",
+                  "paper_2212_10680_gb300/csrc/fmlbm_log.cuh"]
 
 
 # ---- ranks (torchrun): independent problems are split, timings reduced; no data exchange ----
@@ -107,6 +110,20 @@ def measured_peaks() -> dict:
             d = json.load(f)
         return dict(hbm_gbs=float(d["hbm_gbs"]), source="measured")
     return dict(hbm_gbs=6800.0, source="fallback")
+
+
+def step_kernel(variant: str, prec: str, n: int, nodes: int, tile_y: int = 0) -> str:
+    """The kernel that a step runs (the two-launch forms by their second)."""
+    named = {"tma": "fused_step_tma", "tma_tile": "fused_step_tma", "pair": "fused_step_pair", "multi": "fused_steps"}
+    if variant in named:
+        return named[variant]
+    if tile_y not in (0, 8):
+        return "fused_step"
+    if prec == "fp64" or prec.endswith("lnf64"):
+        return "collide_fields"
+    if n in (2, 3) and nodes >= 1 << 19:
+        return "march_step"
+    return "pack_step" if n == 2 and nodes >= 1 << 16 else "fused_step"
 
 
 def profile_traffic(kernel: str, workload_key: str, precision: str):
@@ -468,7 +485,8 @@ def ternary_forms(fmlbm, torch, stream, dev, steps, warmup, flush):
         out[prec] = dict(value=r["n"] * r["nodes"] / per / 1e9, unit="component-GLUPS", ms_per_step=1e3 * per,
                          steps=k, roofline=dict(bound="hbm", achieved=achieved, peak=peak["hbm_gbs"], unit="GB/s",
                                                 frac=achieved / peak["hbm_gbs"],
-                                                traffic=profile_traffic("fused_step", "ternary4096", prec),
+                                                traffic=profile_traffic(step_kernel("plain", prec, r["n"], r["nodes"]),
+                                                                        "ternary4096", prec),
                                                 algorithmic_bytes_per_component_node=ALGO_BYTES[prec]),
                          clocks=r["clocks"])
     return dict(workload=w["name"] + ", tau 1, isotropic, lagged, plain step", forms=out)
@@ -527,8 +545,7 @@ def run_ours(args, w, rank, world, dist):
     algo = ALGO_BYTES[prec] * n * nodes
     peak = measured_peaks()
     achieved = algo / per_launch_s / 1e9
-    kernel_name = {"tma": "fused_step_tma", "tma_tile": "fused_step_tma", "pair": "fused_step_pair"}.get(variant,
-                                                                                                     "fused_step")
+    kernel_name = step_kernel(variant, prec, n, nodes, tuned["tile_y"] if tuned else args.tile_y)
     # the committed counters describe the workload at its own size only
     traffic = None if args.size else profile_traffic(kernel_name, args.workload, prec)
     e2e = _e2e_rate(fmlbm, torch, w, prec, args.steps, stream, dev, dist)

@@ -279,12 +279,16 @@ fmlbm_status fmlbm_set_state(fmlbm_handle* h, const void* buf, size_t bytes);
 
 /* Tuning: height (8, 16 or 32 rows) of the 32-column tile each thread block of the
  * plain fused step owns (moments always use 8 or 16).  Results do not depend on it
- * (bit-identical).  Default: 8 (the fastest measured on GB300 for two and three
- * components; taller tiles recompute less halo but keep fewer blocks per SM). */
+ * (bit-identical).  Default: 8, with which the library takes the fastest form measured on
+ * GB300 for the lattice's size, components and storage: 32 x 8 tiles, with two components
+ * per packed value from 2^16 nodes on (two components), warps that march over the rows from
+ * 2^19 nodes on (two and three components, float and 16-bit storage), or two launches per
+ * step (FP64 and the forms with ln f in FP64; their scratch planes are allocated with the
+ * lattice, and without memory for them the step is one launch). */
 fmlbm_status fmlbm_set_tile_height(fmlbm_handle* h, int32_t tile_y);
 
-/* Which kernel advances the lattice.  PLAIN: the fused step with per-thread pulls from
- * global memory, one node per thread.  PAIR: the same step with two nodes per thread (32
+/* Which kernel advances the lattice.  PLAIN: the step with per-thread pulls from global
+ * memory, one node per thread (see fmlbm_set_tile_height).  PAIR: the same step with two nodes per thread (32
  * columns apart in a 64-column tile) whose float arithmetic runs as packed two-lane
  * instructions; float and 16-bit storage, well-balanced formulation, 8-row tiles.  TMA: a persistent fused step whose blocks copy each wrap-free tile of
  * 32 x 8 nodes (every plane plus a 3-node halo) into shared memory with one bulk tensor
@@ -338,8 +342,9 @@ fmlbm_status fmlbm_set_wait_limit(fmlbm_handle* h, int64_t polls);
  * kernel errors. */
 fmlbm_status fmlbm_synchronize(fmlbm_handle* h);
 
-/* Device bytes one lattice of this shape and precision holds (for admission
- * control). */
+/* Device bytes one lattice of this shape and precision holds (for admission control),
+ * without the scratch planes of a handle's two-launch step and the second density snapshot
+ * that a handle allocates when a large lattice is monitored. */
 fmlbm_status fmlbm_lattice_bytes(int32_t n_components, const fmlbm_lattice* lattice, size_t* bytes);
 
 /* Allocation-free variant of the reductions of fmlbm_diagnostics, for callers that

@@ -175,8 +175,11 @@ cudaError_t launch_split_ty(const StepArgs& A, cudaStream_t s) {
 }
 template <int NC, int ST>
 cudaError_t launch_split(const StepArgs& A, cudaStream_t s) {
-    // Two-row blocks spread a small lattice over the multiprocessors; above 2^16 nodes there are
-    // more 8-row blocks than multiprocessors and the smaller halo counts.
+    // Two-row blocks spread a small lattice over the multiprocessors; from 2^16 nodes on there are
+    // more 8-row blocks than multiprocessors and the smaller halo counts.  us per step, 8 -> 2 rows,
+    // binary FP64: 64^2 29.6 -> 18.3, 128^2 29.8 -> 19.6, 192^2 30.1 -> 31.8, 256^2 54.5 -> 53.7,
+    // 384^2 104 -> 113, 1024^2 672 -> 728; ln f in FP64 over BF16: 64^2 11.2 -> 8.9, 256^2 17.4 -> 17.1,
+    // 384^2 30.8 -> 32.5.
     return (size_t)A.nx * A.ny <= 65536 ? launch_split_ty<NC, ST, 2>(A, s) : launch_split_ty<NC, ST, 8>(A, s);
 }
 
