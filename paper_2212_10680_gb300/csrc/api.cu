@@ -46,6 +46,7 @@ struct fmlbm_handle {
     void* rho_prev = nullptr;     // storage arithmetic type
     int have_prev = 0;
     void* rho_next = nullptr;        // a second snapshot, for steps that write the densities they read
+    bool snap_fixed = false;         // a captured request holds rho_prev's address: the two no longer swap
     void* partial = nullptr;         // kDiagSlots sets of per-strip sums (doubles)
     double* diag_dev = nullptr;      // kDiagSlots x kDiagWords results, then the error latch
     cudaStream_t tail = nullptr;     // final sums and copies of fused requests (non-blocking)
@@ -375,10 +376,12 @@ cudaError_t dispatch_reduce(fmlbm_handle* h, const StepArgs& A, void* partial, d
 
 // Whether a pending request is served by a marching step that writes the densities of the state it
 // reads and a reduction over them (every step of a 1024^2 binary asked: 46.5 us per step, with the
-// sums fused into tile steps 48.5).  Not under capture: the two snapshots swap with every request.
+// sums fused into tile steps 48.5).  Not under capture nor on a handle that served a request under
+// capture: the two snapshots swap with every request, and a replay reads and writes the one it was
+// captured with.
 // The second snapshot comes with the first such step; without memory for it the sums are fused.
-bool serve_by_snapshot(fmlbm_handle* h, const StepArgs& A, bool capturing) {
-    if (capturing || h->tile_y != kTileYSmall || resolved_variant(h) != FMLBM_VARIANT_PLAIN) return false;
+bool serve_by_snapshot(fmlbm_handle* h, const StepArgs& A) {
+    if (h->snap_fixed || h->tile_y != kTileYSmall || resolved_variant(h) != FMLBM_VARIANT_PLAIN) return false;
     bool takes = false;
     switch (h->lattice.precision) {
         case FMLBM_FP32: takes = march_takes<ST_F32>(A, h->nc); break;
@@ -506,6 +509,7 @@ fmlbm_status enqueue_pending_standalone(fmlbm_handle* h) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     FM_CUDA(h, cudaStreamIsCapturing(h->stream, &cap));
     const bool capturing = cap != cudaStreamCaptureStatusNone;
+    h->snap_fixed = h->snap_fixed || capturing;
     if (!capturing) FM_CUDA(h, cudaStreamWaitEvent(h->stream, h->tail_done[t % kDiagSlots], 0));
     FM_CUDA(h, dispatch_reduce(h, A, partial_set(h, t), result_slot(h, t)));
     return enqueue_diag_tail(h, t, h->stream, false, capturing);
@@ -828,12 +832,13 @@ fmlbm_status fmlbm_step(fmlbm_handle* h, int64_t nsteps) {
         bool snapshot = false;
         A.pdl = A.pdl_chain = pdl;
         if (fused >= 0) {  // this step also reduces the state it reads
+            h->snap_fixed = h->snap_fixed || capturing;
             // the tail of request fused - kDiagSlots may still read this set of partial sums
             if (!capturing && h->tail_open[fused % kDiagSlots]) {
                 FM_CUDA(h, cudaStreamWaitEvent(h->stream, h->tail_done[fused % kDiagSlots], 0));
                 A.pdl = 0;
             }
-            snapshot = serve_by_snapshot(h, A, capturing);
+            snapshot = serve_by_snapshot(h, A);
             if (snapshot) {
                 A.rho_snap = h->rho_next;
             } else {

@@ -1,0 +1,77 @@
+"""Steps captured into a graph and replayed between launched calls: the same state, diagnostics and
+counts as stepping directly."""
+import numpy as np
+import pytest
+
+from cases import mixture_dict, smooth_state
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fm():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2212_10680_gb300 import fmlbm
+    return fmlbm
+
+
+def _capture(stream, call):
+    import torch
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+        call()
+
+    def replay(times=1):
+        with torch.cuda.stream(stream):
+            for _ in range(times):
+                graph.replay()
+        stream.synchronize()
+    return replay
+
+
+@pytest.mark.parametrize("precision,n,shape", [("fp32", 2, (1024, 512)), ("bf16dev", 3, (1024, 512)),
+                                               ("fp32", 2, (300, 256)), ("fp64", 2, (70, 45))])
+def test_requests_captured_and_launched_share_one_snapshot(fm, precision, n, shape):
+    # every residual is taken against the state of the request before it, whether a replayed graph or a
+    # launched step served that one (2^19 nodes: the marching step; then packed tiles and the split step)
+    import torch
+    nx, ny = shape
+    mixd = mixture_dict(n, "pr", Tr=0.9, kappa_scale=0.3)
+    rho = smooth_state(n, nx, ny, seed=3)
+
+    def lattice(stream):
+        lat = fm.Lattice(fm.mixture_from_dict(mixd), nx, ny, 0.9, "isotropic", precision, "lagged", stream=stream)
+        lat.init(rho)
+        fm.fmlbm_synchronize(lat.h)
+        return lat
+
+    ref, expect = lattice(0), []
+    for _ in range(5):
+        expect.append(ref.diagnostics()[:2])
+        ref.step(2)
+    s = torch.cuda.Stream()
+    lat, got = lattice(s.cuda_stream), []
+
+    def launched():
+        t = fm.fmlbm_diagnostics_async(lat.h)
+        lat.step(2)
+        got.append(fm.fmlbm_diagnostics_wait(lat.h, t, n)[:2])
+        fm.fmlbm_synchronize(lat.h)
+
+    launched()
+    ticket = fm.fmlbm_diagnostics_async(lat.h)
+    replay = _capture(s, lambda: lat.step(2))
+
+    def replayed():
+        replay()
+        got.append(fm.fmlbm_diagnostics_wait(lat.h, ticket, n)[:2])
+
+    for serve in (replayed, launched, replayed, launched):
+        serve()
+    for k, ((mass, res), (mass_ref, res_ref)) in enumerate(zip(got, expect)):
+        assert np.array_equal(mass, mass_ref) and res == res_ref, k
+    for u, v in zip(lat.distributions(), ref.distributions()):
+        assert np.array_equal(u, v)
+    lat.close()
+    ref.close()
