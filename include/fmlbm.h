@@ -411,7 +411,10 @@ fmlbm_status fmlbm_batch_add(fmlbm_batch* b, const fmlbm_mixture* mixture, const
 fmlbm_status fmlbm_batch_remove(fmlbm_batch* b, int32_t slot);
 /* Pauses (0) or resumes (1) stepping of a slot. */
 fmlbm_status fmlbm_batch_set_active(fmlbm_batch* b, int32_t slot, int32_t active);
-/* Enqueues nsteps steps of every active slot (asynchronous). */
+/* Enqueues nsteps steps of every active slot (asynchronous).  While the batch's stream is being
+ * captured the steps become part of the graph: each replay of it takes them, and the calls below
+ * that report or read a slot (which then wait for the batch's stream) count them.  Replay it only
+ * while the slots that were active at the capture are the active ones. */
 fmlbm_status fmlbm_batch_step(fmlbm_batch* b, int64_t nsteps);
 /* Residual and error check of every active slot (synchronises); results via
  * fmlbm_batch_slot_info.  The first check after a slot is added sets its snapshot

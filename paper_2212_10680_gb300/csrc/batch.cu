@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <new>
 #include <string>
@@ -27,7 +28,8 @@ struct Slot {
     float* g0[2] = {nullptr, nullptr};
     void* F[2] = {nullptr, nullptr};
     void* prev = nullptr;     // density snapshot, storage arithmetic type
-    long long steps = 0;      // host mirror of the device counter
+    long long steps = 0;      // host mirror of the device counter (behind it after replays: read_counts)
+    bool uploaded = false;    // has its counter on the device
     bool have_prev = false;
     double residual = INFINITY;
     double lam[kMaxC] = {};          // phase measure at the last check: mean of ln rho_i
@@ -64,7 +66,7 @@ struct fmlbm_batch {
     // launches of one packed step: [steps enqueued since they were made & 1]
     std::vector<PackGroup> groups[2];
     long long since = 0;
-    bool counted = false;       // a captured step's replays have their counts on the device only
+    bool captured = false;      // steps were captured: replays of them advance the device's counters only
     void** d_prev = nullptr;
     double* d_partial = nullptr;
     int partial_cap = 0;
@@ -136,7 +138,7 @@ template <int ST, int NC>
 cudaError_t launch_batch_step_nc(const fmlbm_batch* b, int ahead, bool pdl) {
     if (b->tile_y == kTileYLarge) return launch_batch_step_t<ST, NC, kTileYLarge>(b, ahead, pdl);
     if constexpr (NC == 2 && kSpecStep<ST>) {
-        if (!b->counted) return b->spec ? launch_batch_pack<ST, true>(b, ahead, pdl) : launch_batch_pack<ST, false>(b, ahead, pdl);
+        if (!b->captured) return b->spec ? launch_batch_pack<ST, true>(b, ahead, pdl) : launch_batch_pack<ST, false>(b, ahead, pdl);
     }
     return launch_batch_step_t<ST, NC, kTileYSmall>(b, ahead, pdl);
 }
@@ -223,12 +225,11 @@ void fill_descriptor(fmlbm_batch* b, int k) {
 // The packed step's parameters of the active slots, for both parities.
 void fill_groups(fmlbm_batch* b) {
     b->since = 0;
-    b->counted = false;
     const bool dev16 = b->precision != FMLBM_FP32;
     for (int p = 0; p < 2; ++p) {
         std::vector<PackGroup>& gs = b->groups[p];
         gs.clear();
-        if (!packed(b)) continue;
+        if (!packed(b) || b->captured) continue;
         for (int k = 0; k < b->capacity; ++k) {
             const Slot& s = b->slots[k];
             if (!s.used || !s.active) continue;
@@ -255,9 +256,28 @@ void fill_groups(fmlbm_batch* b) {
     }
 }
 
+// The step counts after replays of captured steps, which advance the counters on the device only
+// (synchronises; not during a capture, whose steps count when they are replayed).
+fmlbm_status read_counts(fmlbm_batch* b) {
+    if (!b->captured) return FMLBM_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    BCUDA(b, cudaStreamIsCapturing(b->stream, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return FMLBM_OK;
+    std::vector<long long> n(b->capacity);
+    BCUDA(b, cudaMemcpy2DAsync(n.data(), sizeof(long long),
+                               reinterpret_cast<const char*>(b->d_lat) + offsetof(BatchLattice, step),
+                               sizeof(BatchLattice), sizeof(long long), b->capacity, cudaMemcpyDeviceToHost, b->stream));
+    BCUDA(b, cudaStreamSynchronize(b->stream));
+    for (int k = 0; k < b->capacity; ++k)
+        if (b->slots[k].used && b->slots[k].uploaded) b->slots[k].steps = n[k];
+    return FMLBM_OK;
+}
+
 // Rebuild the work list (active slots only, items of a slot contiguous) and upload the
 // descriptors.
 fmlbm_status rebuild(fmlbm_batch* b) {
+    fmlbm_status st = read_counts(b);
+    if (st != FMLBM_OK) return st;
     std::vector<WorkItem> items;
     b->spec = true;
     for (int k = 0; k < b->capacity; ++k) {
@@ -292,6 +312,7 @@ fmlbm_status rebuild(fmlbm_batch* b) {
     for (int k = 0; k < b->capacity; ++k) prev[k] = b->slots[k].prev;
     BCUDA(b, cudaMemcpyAsync(b->d_prev, prev.data(), prev.size() * sizeof(void*), cudaMemcpyHostToDevice, b->stream));
     BCUDA(b, cudaStreamSynchronize(b->stream));  // host vectors above are temporaries
+    for (Slot& s : b->slots) s.uploaded = s.used;
     b->work_dirty = false;
     return FMLBM_OK;
 }
@@ -300,13 +321,13 @@ fmlbm_status ensure_work(fmlbm_batch* b) { return b->work_dirty ? rebuild(b) : F
 
 // Enqueue n steps of all active slots (no synchronisation), launched programmatically behind one
 // another (serving 12 lattices of 64^2 to 184^2 took 26.0 ms with the launches of a check interval
-// captured in a graph, 24.0 ms with these).  Steps under stream capture, and those after them until
-// the next rebuild, choose their buffers by the counters on the device, which a replay advances.
+// captured in a graph, 24.0 ms with these).  Steps under stream capture, and all of the batch's steps
+// from then on, choose their buffers by the counters on the device, which a replay advances.
 fmlbm_status enqueue_steps(fmlbm_batch* b, long long n) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     BCUDA(b, cudaStreamIsCapturing(b->stream, &cap));
     const bool capturing = cap != cudaStreamCaptureStatusNone;
-    b->counted = b->counted || capturing;
+    b->captured = b->captured || capturing;
     const int nb = (b->capacity + 127) / 128;
     for (long long done = 0; done < n;) {
         const int m = (int)std::min<long long>(n - done, 1 << 20);
@@ -317,7 +338,7 @@ fmlbm_status enqueue_steps(fmlbm_batch* b, long long n) {
         done += m;
     }
     for (auto& s : b->slots)
-        if (s.used && s.active) s.steps += n;
+        if (s.used && s.active && !capturing) s.steps += n;
     return FMLBM_OK;
 }
 
@@ -572,7 +593,8 @@ fmlbm_status fmlbm_batch_step(fmlbm_batch* b, int64_t nsteps) {
 fmlbm_status fmlbm_batch_run(fmlbm_batch* b, int64_t max_steps, int32_t check_every, double tol, int64_t* steps_out,
                              double* residual_out, int32_t* status_out) {
     if (!b || max_steps < 0 || check_every < 1) return bfail(b, FMLBM_E_INVALID_ARG, "bad argument");
-    fmlbm_status st = ensure_work(b);
+    fmlbm_status st = read_counts(b);
+    if (st == FMLBM_OK) st = ensure_work(b);
     if (st != FMLBM_OK) return st;
     // first snapshot of every active slot
     st = check_all(b);
@@ -629,6 +651,8 @@ fmlbm_status fmlbm_batch_run_chunk(fmlbm_batch* b, int32_t steps) {
 fmlbm_status fmlbm_batch_slot_info(fmlbm_batch* b, int32_t slot, int64_t* steps, double* residual, int32_t* status,
                                    int32_t* active) {
     if (!b || slot < 0 || slot >= b->capacity || !b->slots[slot].used) return bfail(b, FMLBM_E_INVALID_ARG, "bad slot");
+    const fmlbm_status st = read_counts(b);
+    if (st != FMLBM_OK) return st;
     const Slot& s = b->slots[slot];
     if (steps) *steps = s.steps;
     if (residual) *residual = s.residual;
@@ -660,6 +684,8 @@ fmlbm_status fmlbm_batch_check(fmlbm_batch* b) {
 
 fmlbm_status fmlbm_batch_moments(fmlbm_batch* b, int32_t slot, double* rho, double* u, double* lnf) {
     if (!b || slot < 0 || slot >= b->capacity || !b->slots[slot].used) return bfail(b, FMLBM_E_INVALID_ARG, "bad slot");
+    const fmlbm_status st = read_counts(b);
+    if (st != FMLBM_OK) return st;
     Slot& s = b->slots[slot];
     const size_t nxy = (size_t)s.L.nx * s.L.ny;
     const size_t fb = (size_t)b->nc * nxy * sizeof(double);
@@ -678,6 +704,8 @@ fmlbm_status fmlbm_batch_moments(fmlbm_batch* b, int32_t slot, double* rho, doub
 
 fmlbm_status fmlbm_batch_phases(fmlbm_batch* b, int32_t slot, double* rho_liquid, double* rho_vapour) {
     if (!b || slot < 0 || slot >= b->capacity || !b->slots[slot].used) return bfail(b, FMLBM_E_INVALID_ARG, "bad slot");
+    const fmlbm_status st = read_counts(b);
+    if (st != FMLBM_OK) return st;
     Slot& s = b->slots[slot];
     const size_t nxy = (size_t)s.L.nx * s.L.ny;
     double* d = nullptr;
@@ -709,6 +737,8 @@ fmlbm_status fmlbm_batch_phases(fmlbm_batch* b, int32_t slot, double* rho_liquid
 
 fmlbm_status fmlbm_batch_get_distributions(fmlbm_batch* b, int32_t slot, double* g, double* force) {
     if (!b || slot < 0 || slot >= b->capacity || !b->slots[slot].used) return bfail(b, FMLBM_E_INVALID_ARG, "bad slot");
+    const fmlbm_status st = read_counts(b);
+    if (st != FMLBM_OK) return st;
     Slot& s = b->slots[slot];
     fill_descriptor(b, slot);
     const StepArgs A = b->h_lat[slot].args[s.steps & 1];

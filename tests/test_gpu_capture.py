@@ -3,7 +3,7 @@ counts as stepping directly."""
 import numpy as np
 import pytest
 
-from cases import mixture_dict, smooth_state
+from cases import mixture_dict, slab_state_binary, smooth_state
 
 pytestmark = pytest.mark.gpu
 
@@ -75,3 +75,52 @@ def test_requests_captured_and_launched_share_one_snapshot(fm, precision, n, sha
         assert np.array_equal(u, v)
     lat.close()
     ref.close()
+
+
+def _batch(fm, stream, precision="fp32", shape=(70, 45)):
+    mixd, rho = slab_state_binary(*shape, seed=3)
+    L = fm.make_lattice(*shape, 1.0, precision=precision)
+    b = fm.fmlbm_batch_create(2, precision, 3, stream.cuda_stream)
+    return b, fm.fmlbm_batch_add(b, fm.mixture_from_dict(mixd), L, rho), (mixd, rho, precision)
+
+
+def _after(fm, b, slot, case, steps):
+    """Whether the slot's state, fields, phases and count are those of the same lattice after `steps` steps."""
+    mixd, rho, precision = case
+    n, ny, nx = rho.shape
+    lat = fm.Lattice(fm.mixture_from_dict(mixd), nx, ny, 1.0, precision=precision)
+    lat.init(rho)
+    lat.step(steps)
+    want = lat.distributions() + (lat.moments()[0],)
+    lat.close()
+    got = np.empty((n, 9, ny, nx)), np.empty((2, ny, nx)), np.empty((n, ny, nx))
+    fm.fmlbm_batch_moments(b, slot, got[2])
+    fm.fmlbm_batch_get_distributions(b, slot, *got[:2])
+    liquid, vapour = fm.fmlbm_batch_phases(b, slot, n)
+    return (all(np.array_equal(u, v) for u, v in zip(got, want)) and liquid.sum() > vapour.sum() and
+            fm.fmlbm_batch_slot_info(b, slot)[0] == steps)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])   # packed tiles; the batch kernel alone
+@pytest.mark.parametrize("rebuild", [False, True])
+@pytest.mark.parametrize("replays", [0, 1, 2, 3])
+def test_batch_counts_the_replays_of_captured_steps(fm, precision, rebuild, replays):
+    import torch
+    s = torch.cuda.Stream()
+    b, slot, case = _batch(fm, s, precision)
+    fm.fmlbm_batch_step(b, 1)
+    s.synchronize()
+    replay = _capture(s, lambda: fm.fmlbm_batch_step(b, 1))
+    if rebuild:   # descriptors and counters are uploaded again
+        fm.fmlbm_batch_set_active(b, slot, False)
+        fm.fmlbm_batch_set_active(b, slot, True)
+    fm.fmlbm_batch_step(b, 1)
+    replay(replays)
+    assert _after(fm, b, slot, case, 2 + replays)
+    fm.fmlbm_batch_step(b, 1)
+    replay()
+    assert _after(fm, b, slot, case, 4 + replays)
+    steps, _, _ = fm.fmlbm_batch_run(b, 3, max_steps=9 + replays, check_every=5, tol=0.0)
+    assert steps[slot] == 9 + replays
+    assert _after(fm, b, slot, case, 9 + replays)
+    fm.fmlbm_batch_destroy(b)
