@@ -342,6 +342,14 @@ fmlbm_status enqueue_steps(fmlbm_batch* b, long long n) {
     return FMLBM_OK;
 }
 
+// Calls that wait for the stream are refused while it is being captured, before they put anything
+// into the graph or count it.
+fmlbm_status refuse_capture(fmlbm_batch* b) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    BCUDA(b, cudaStreamIsCapturing(b->stream, &cap));
+    return cap == cudaStreamCaptureStatusNone ? FMLBM_OK : bfail(b, FMLBM_E_CUDA, "the batch's stream is being captured");
+}
+
 // Reductions of every active slot -> residuals and phase-measure changes; latched errors ->
 // statuses.  Synchronises.
 fmlbm_status check_all(fmlbm_batch* b) {
@@ -593,7 +601,8 @@ fmlbm_status fmlbm_batch_step(fmlbm_batch* b, int64_t nsteps) {
 fmlbm_status fmlbm_batch_run(fmlbm_batch* b, int64_t max_steps, int32_t check_every, double tol, int64_t* steps_out,
                              double* residual_out, int32_t* status_out) {
     if (!b || max_steps < 0 || check_every < 1) return bfail(b, FMLBM_E_INVALID_ARG, "bad argument");
-    fmlbm_status st = read_counts(b);
+    fmlbm_status st = refuse_capture(b);
+    if (st == FMLBM_OK) st = read_counts(b);
     if (st == FMLBM_OK) st = ensure_work(b);
     if (st != FMLBM_OK) return st;
     // first snapshot of every active slot
@@ -641,7 +650,8 @@ fmlbm_status fmlbm_batch_run(fmlbm_batch* b, int64_t max_steps, int32_t check_ev
 
 fmlbm_status fmlbm_batch_run_chunk(fmlbm_batch* b, int32_t steps) {
     if (!b || steps < 1) return bfail(b, FMLBM_E_INVALID_ARG, "bad argument");
-    fmlbm_status st = ensure_work(b);
+    fmlbm_status st = refuse_capture(b);
+    if (st == FMLBM_OK) st = ensure_work(b);
     if (st != FMLBM_OK || b->nwork == 0) return st;
     st = enqueue_steps(b, steps);
     if (st != FMLBM_OK) return st;

@@ -124,3 +124,27 @@ def test_batch_counts_the_replays_of_captured_steps(fm, precision, rebuild, repl
     assert steps[slot] == 9 + replays
     assert _after(fm, b, slot, case, 9 + replays)
     fm.fmlbm_batch_destroy(b)
+
+
+@pytest.mark.parametrize("call", ["chunk", "run"])
+def test_batch_runs_are_refused_under_capture_and_leave_no_trace(fm, call):
+    import torch
+    s = torch.cuda.Stream()
+    b, slot, case = _batch(fm, s)
+    fm.fmlbm_batch_step(b, 2)
+    s.synchronize()
+
+    def refused():
+        with pytest.raises(fm.FmlbmError) as e:
+            if call == "chunk":
+                fm.fmlbm_batch_run_chunk(b, 3)
+            else:
+                fm.fmlbm_batch_run(b, 3, max_steps=5, check_every=3, tol=0.0)
+        assert e.value.status == 3   # FMLBM_E_CUDA
+        fm.fmlbm_batch_step(b, 1)   # the capture goes on
+
+    replay = _capture(s, refused)
+    assert _after(fm, b, slot, case, 2)
+    replay()
+    assert _after(fm, b, slot, case, 3)
+    fm.fmlbm_batch_destroy(b)
