@@ -147,7 +147,9 @@ typedef struct fmlbm_handle fmlbm_handle;
 
 /* Creates a lattice: validates the mixture (Appendix C parameters) and lattice,
  * allocates its device buffers (two distribution buffers, two force buffers,
- * a density snapshot for the residual and reduction scratch) and a second stream for
+ * a density snapshot for the residual and reduction scratch; where there is memory for them also
+ * the scratch planes of a two-launch step and the second snapshot of a marching one, see
+ * fmlbm_set_tile_height) and a second stream for
  * diagnostics on the current device, and leaves it uninitialised.  cuda_stream: a cudaStream_t (may be
  * NULL), owned by the caller, must outlive the handle. */
 fmlbm_status fmlbm_create(const fmlbm_mixture* mixture, const fmlbm_lattice* lattice,
@@ -282,7 +284,8 @@ fmlbm_status fmlbm_set_state(fmlbm_handle* h, const void* buf, size_t bytes);
  * (bit-identical).  Default: 8, with which the library takes the fastest form measured on
  * GB300 for the lattice's size, components and storage: 32 x 8 tiles, with two components
  * per packed value from 2^16 nodes on (two components), warps that march over the rows from
- * 2^19 nodes on (two and three components, float and 16-bit storage), or two launches per
+ * 2^19 nodes on (two and three components, float and 16-bit storage; a second density snapshot,
+ * for their diagnostics, is allocated with the lattice), or two launches per
  * step (FP64 and the forms with ln f in FP64; their scratch planes are allocated with the
  * lattice, and without memory for them the step is one launch). */
 fmlbm_status fmlbm_set_tile_height(fmlbm_handle* h, int32_t tile_y);
@@ -344,7 +347,7 @@ fmlbm_status fmlbm_synchronize(fmlbm_handle* h);
 
 /* Device bytes one lattice of this shape and precision holds (for admission control),
  * without the scratch planes of a handle's two-launch step and the second density snapshot
- * that a handle allocates when a large lattice is monitored. */
+ * of a large lattice. */
 fmlbm_status fmlbm_lattice_bytes(int32_t n_components, const fmlbm_lattice* lattice, size_t* bytes);
 
 /* Allocation-free variant of the reductions of fmlbm_diagnostics, for callers that

@@ -45,7 +45,7 @@ struct fmlbm_handle {
     int cur = 0;
     void* rho_prev = nullptr;     // storage arithmetic type
     int have_prev = 0;
-    void* rho_next = nullptr;        // a second snapshot, for steps that write the densities they read
+    void* rho_next = nullptr;        // a second snapshot, for marching steps that write the densities they read
     bool snap_fixed = false;         // a captured request holds rho_prev's address: the two no longer swap
     void* partial = nullptr;         // kDiagSlots sets of per-strip sums (doubles)
     double* diag_dev = nullptr;      // kDiagSlots x kDiagWords results, then the error latch
@@ -379,27 +379,10 @@ cudaError_t dispatch_reduce(fmlbm_handle* h, const StepArgs& A, void* partial, d
 // sums fused into tile steps 48.5).  Not under capture nor on a handle that served a request under
 // capture: the two snapshots swap with every request, and a replay reads and writes the one it was
 // captured with.
-// The second snapshot comes with the first such step; without memory for it the sums are fused.
-bool serve_by_snapshot(fmlbm_handle* h, const StepArgs& A) {
-    if (h->snap_fixed || h->tile_y != kTileYSmall || resolved_variant(h) != FMLBM_VARIANT_PLAIN) return false;
-    bool takes = false;
-    switch (h->lattice.precision) {
-        case FMLBM_FP32: takes = march_takes<ST_F32>(A, h->nc); break;
-        case FMLBM_FP16DEV: takes = march_takes<ST_F16DEV>(A, h->nc); break;
-        case FMLBM_BF16DEV: takes = march_takes<ST_BF16DEV>(A, h->nc); break;
-        default: break;
-    }
-    if (takes && !h->rho_next) {
-        // a stream capture in global mode elsewhere forbids every thread to allocate
-        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-        cudaThreadExchangeStreamCaptureMode(&mode);
-        if (cudaMalloc(&h->rho_next, (size_t)h->nc * h->lattice.nx * h->lattice.ny * sizeof(float)) != cudaSuccess) {
-            cudaGetLastError();
-            h->rho_next = nullptr;
-        }
-        cudaThreadExchangeStreamCaptureMode(&mode);
-    }
-    return takes && h->rho_next;
+// The second snapshot is allocated with a lattice that marches; without memory for it the sums are
+// fused.
+bool serve_by_snapshot(const fmlbm_handle* h) {
+    return h->rho_next && !h->snap_fixed && h->tile_y == kTileYSmall && resolved_variant(h) == FMLBM_VARIANT_PLAIN;
 }
 
 cudaError_t dispatch_lnrho(fmlbm_handle* h, const StepArgs& A, double* partial, double* out) {
@@ -541,6 +524,20 @@ PFN_cuMemGetAddressRange_v3020 address_range_fn() {
     return fn;
 }
 
+// Whether the plain step of this lattice marches (on 8-row tiles).
+bool marches(int nc, const fmlbm_lattice& L) {
+    StepArgs A{};
+    A.nx = L.nx;
+    A.ny = L.ny;
+    A.standard = L.formulation == FMLBM_STANDARD;
+    switch (L.precision) {
+        case FMLBM_FP32: return march_takes<ST_F32>(A, nc);
+        case FMLBM_FP16DEV: return march_takes<ST_F16DEV>(A, nc);
+        case FMLBM_BF16DEV: return march_takes<ST_BF16DEV>(A, nc);
+        default: return false;
+    }
+}
+
 // Byte ranges [p, p + bytes) that must not overlap (null entries are skipped).
 bool disjoint(const void* const* p, const size_t* bytes, int n) {
     for (int i = 0; i < n; ++i)
@@ -640,6 +637,10 @@ fmlbm_status create_handle(const fmlbm_mixture* mixture, const fmlbm_lattice* la
         cudaMalloc(&h->fields, split_planes(h->nc, f64) * nxy * real_size(lattice->precision)) != cudaSuccess) {
         cudaGetLastError();
         h->fields = nullptr;
+    }
+    if (marches(h->nc, *lattice) && cudaMalloc(&h->rho_next, h->nc * nxy * sizeof(float)) != cudaSuccess) {
+        cudaGetLastError();
+        h->rho_next = nullptr;
     }
     setup_tma(h);
     *out = h;
@@ -838,7 +839,7 @@ fmlbm_status fmlbm_step(fmlbm_handle* h, int64_t nsteps) {
                 FM_CUDA(h, cudaStreamWaitEvent(h->stream, h->tail_done[fused % kDiagSlots], 0));
                 A.pdl = 0;
             }
-            snapshot = serve_by_snapshot(h, A);
+            snapshot = serve_by_snapshot(h);
             if (snapshot) {
                 A.rho_snap = h->rho_next;
             } else {

@@ -1,0 +1,48 @@
+"""Device memory of a handle: what it holds, and that stepping takes none."""
+import numpy as np
+import pytest
+
+from cases import mixture_dict, smooth_state
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fm():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2212_10680_gb300 import fmlbm
+    return fmlbm
+
+
+def _free():
+    import torch
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+def _lattice(fm, n, nx, ny, precision):
+    lat = fm.Lattice(fm.mixture_from_dict(mixture_dict(n, Tr=0.9, kappa_scale=0.3)), nx, ny, 0.9, precision=precision)
+    lat.init(smooth_state(n, nx, ny, seed=1))
+    return lat
+
+
+def _monitored(fm, lat, n):
+    fm.fmlbm_diagnostics_wait(lat.h, fm.fmlbm_diagnostics_async(lat.h), n)
+    t = fm.fmlbm_diagnostics_async(lat.h)
+    lat.step(1)
+    fm.fmlbm_diagnostics_wait(lat.h, t, n)
+    lat.synchronize()
+
+
+@pytest.mark.parametrize("n,precision,shape", [(2, "fp32", (2048, 1024)), (3, "bf16dev", (2048, 1024)),
+                                               (2, "fp64", (512, 512))])
+def test_a_monitored_step_allocates_nothing(fm, n, precision, shape):
+    # the first lattice loads every kernel of the run; 16 MB and more in question for the second
+    first, second = (_lattice(fm, n, *shape, precision) for _ in range(2))
+    _monitored(fm, first, n)
+    before = _free()
+    _monitored(fm, second, n)
+    assert _free() == before
+    first.close()
+    second.close()
