@@ -345,9 +345,10 @@ fmlbm_status fmlbm_set_wait_limit(fmlbm_handle* h, int64_t polls);
  * kernel errors. */
 fmlbm_status fmlbm_synchronize(fmlbm_handle* h);
 
-/* Device bytes one lattice of this shape and precision holds (for admission control),
- * without the scratch planes of a handle's two-launch step and the second density snapshot
- * of a large lattice. */
+/* Device bytes one lattice of this shape and precision holds (for admission control), with
+ * the scratch planes of a two-launch step and the second density snapshot of a marching one,
+ * which only a handle has (a batch's lattice does without) and without which it steps in another
+ * form: see fmlbm_set_tile_height. */
 fmlbm_status fmlbm_lattice_bytes(int32_t n_components, const fmlbm_lattice* lattice, size_t* bytes);
 
 /* Allocation-free variant of the reductions of fmlbm_diagnostics, for callers that
@@ -474,7 +475,7 @@ fmlbm_status fmlbm_batch_phases(fmlbm_batch* b, int32_t slot, double* rho_liquid
  * Serving: vapour-liquid solves submitted as requests and run with continuous batching.
  * A worker thread owns a batch; between chunks of chunk_steps steps it admits queued
  * requests in arrival order while a slot is free and their device bytes
- * (fmlbm_lattice_bytes) fit hbm_budget_bytes, and retires each running lattice at its
+ * (fmlbm_lattice_bytes without a handle's scratch) fit hbm_budget_bytes, and retires each running lattice at its
  * own criterion (the configured convergence measure < tol at a check, a latched error, or
  * max_steps).  A request's
  * result does not depend on what else is running.  All server functions are

@@ -538,6 +538,17 @@ bool marches(int nc, const fmlbm_lattice& L) {
     }
 }
 
+// Device bytes a handle takes where it can get them: the split step's planes, the second density
+// snapshot of a marching lattice.
+size_t scratch_bytes(int nc, const fmlbm_lattice& L) {
+    const size_t nxy = (size_t)L.nx * (size_t)L.ny;
+    const bool f64 = L.precision == FMLBM_FP64;
+    if ((f64 || L.precision == FMLBM_FP16DEV_LNF64 || L.precision == FMLBM_BF16DEV_LNF64) &&
+        L.formulation == FMLBM_WELL_BALANCED)
+        return split_planes(nc, f64) * nxy * real_size(L.precision);
+    return marches(nc, L) ? nc * nxy * sizeof(float) : 0;
+}
+
 // Byte ranges [p, p + bytes) that must not overlap (null entries are skipped).
 bool disjoint(const void* const* p, const size_t* bytes, int n) {
     for (int i = 0; i < n; ++i)
@@ -630,17 +641,13 @@ fmlbm_status create_handle(const fmlbm_mixture* mixture, const fmlbm_lattice* la
         return FMLBM_E_CUDA;
     }
     cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
-    // the split step's planes; without them (no memory left) the lattice steps fused
-    const bool f64 = lattice->precision == FMLBM_FP64;
-    if ((f64 || lattice->precision == FMLBM_FP16DEV_LNF64 || lattice->precision == FMLBM_BF16DEV_LNF64) &&
-        lattice->formulation == FMLBM_WELL_BALANCED &&
-        cudaMalloc(&h->fields, split_planes(h->nc, f64) * nxy * real_size(lattice->precision)) != cudaSuccess) {
-        cudaGetLastError();
-        h->fields = nullptr;
-    }
-    if (marches(h->nc, *lattice) && cudaMalloc(&h->rho_next, h->nc * nxy * sizeof(float)) != cudaSuccess) {
-        cudaGetLastError();
-        h->rho_next = nullptr;
+    // without memory for these the lattice steps fused, and requests are served by fused sums
+    if (const size_t bytes = scratch_bytes(h->nc, *lattice)) {
+        void** p = marches(h->nc, *lattice) ? &h->rho_next : &h->fields;
+        if (cudaMalloc(p, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            *p = nullptr;
+        }
     }
     setup_tma(h);
     *out = h;
@@ -681,6 +688,12 @@ void fmlbm_internal_set_check_rows(fmlbm_handle* h, int y0, int y1) {
 bool fmlbm_internal_mixture_constants(const fmlbm_mixture& m, MixConst* mc, std::string* why) {
     return mixture_constants(m, mc, why);
 }
+size_t fmlbm_internal_batched_bytes(int nc, const fmlbm_lattice& L) {
+    size_t gb, g0b, fb;
+    buffer_bytes(nc, L, &gb, &g0b, &fb);
+    return 2 * (gb + g0b + fb) + (size_t)nc * L.nx * L.ny * real_size(L.precision) +
+           kDiagSlots * (size_t)reduce_blocks(L.nx, L.ny) * (FMLBM_MAX_COMPONENTS + 2) * 8 + 512;
+}
 bool fmlbm_internal_lattice_ok(const fmlbm_lattice& L, int nc, std::string* why) { return lattice_ok(L, nc, why); }
 
 extern "C" {
@@ -706,11 +719,7 @@ const char* fmlbm_last_error(const fmlbm_handle* h) { return h ? h->last_error.c
 
 fmlbm_status fmlbm_lattice_bytes(int32_t n_components, const fmlbm_lattice* lattice, size_t* bytes) {
     if (!lattice || !bytes || n_components < 1 || n_components > FMLBM_MAX_COMPONENTS) return FMLBM_E_INVALID_ARG;
-    size_t gb, g0b, fb;
-    buffer_bytes(n_components, *lattice, &gb, &g0b, &fb);
-    const size_t nxy = (size_t)lattice->nx * lattice->ny;
-    *bytes = 2 * (gb + g0b + fb) + (size_t)n_components * nxy * real_size(lattice->precision) +
-             kDiagSlots * (size_t)reduce_blocks(lattice->nx, lattice->ny) * (FMLBM_MAX_COMPONENTS + 2) * 8 + 512;
+    *bytes = fmlbm_internal_batched_bytes(n_components, *lattice) + scratch_bytes(n_components, *lattice);
     return FMLBM_OK;
 }
 

@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 
 #include "fmlbm.h"
+#include "fmlbm_internal.h"
 
 namespace {
 
@@ -214,8 +215,7 @@ fmlbm_status fmlbm_server_submit(fmlbm_server* s, const fmlbm_request* req, uint
     if (!s || !req || !req->rho) return FMLBM_E_INVALID_ARG;
     if (req->mixture.n_components != s->cfg.n_components || req->lattice.precision != s->cfg.precision)
         return FMLBM_E_INVALID_ARG;
-    size_t bytes = 0;
-    if (fmlbm_lattice_bytes(req->mixture.n_components, &req->lattice, &bytes) != FMLBM_OK) return FMLBM_E_INVALID_ARG;
+    const size_t bytes = fmlbm_internal_batched_bytes(req->mixture.n_components, req->lattice);
     if (bytes > s->cfg.hbm_budget_bytes) return FMLBM_E_INVALID_ARG;  // could never be admitted
     Pending p;
     p.tag = req->tag;

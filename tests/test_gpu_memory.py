@@ -46,3 +46,32 @@ def test_a_monitored_step_allocates_nothing(fm, n, precision, shape):
     assert _free() == before
     first.close()
     second.close()
+
+
+@pytest.mark.parametrize("n,precision,shape", [(2, "fp64", (1024, 1024)), (3, "bf16dev_lnf64", (2048, 1024)),
+                                               (2, "fp32", (4096, 2048)), (3, "fp16dev", (3000, 2001)),
+                                               (2, "fp32", (512, 512))])
+def test_lattice_bytes_cover_what_a_handle_holds(fm, n, precision, shape):
+    _lattice(fm, n, *shape, precision).close()   # loads the kernels
+    nbytes = fm.fmlbm_lattice_bytes(n, fm.make_lattice(*shape, 0.9, precision=precision))
+    before = _free()
+    lat = _lattice(fm, n, *shape, precision)
+    # ten allocations, each rounded up to 2 MiB
+    assert before - _free() <= nbytes + 10 * (2 << 20)
+    lat.close()
+
+
+def test_a_server_admits_by_what_its_batch_holds(fm):
+    # FP64: a handle's eight scratch planes per node are no part of a served lattice
+    L = fm.make_lattice(64, 64, 1.0, precision="fp64")
+    rho = np.stack([np.full((64, 64), 1.0), np.full((64, 64), 0.8)])
+    need = fm.fmlbm_lattice_bytes(2, L) - 8 * 8 * 64 * 64
+    mix = fm.mixture_from_dict(mixture_dict(2, Tr=1.1, kappa_scale=0.5))
+    for budget, accepted in ((need, True), (need - 1, False)):
+        s = fm.fmlbm_server_create(2, "fp64", 2, 100, 1e-12, 1000, budget)
+        if accepted:
+            fm.fmlbm_server_submit(s, mix, L, rho)
+        else:
+            with pytest.raises(fm.FmlbmError):
+                fm.fmlbm_server_submit(s, mix, L, rho)
+        fm.fmlbm_server_destroy(s)
