@@ -375,12 +375,12 @@ cudaError_t dispatch_reduce(fmlbm_handle* h, const StepArgs& A, void* partial, d
 }
 
 // Whether a pending request is served by a marching step that writes the densities of the state it
-// reads and a reduction over them (every step of a 1024^2 binary asked: 46.5 us per step, with the
-// sums fused into tile steps 48.5).  Not under capture nor on a handle that served a request under
+// reads and a reduction over them (every step of a 1024^2 binary asked: 46.0 us per step, with the
+// sums fused into tile steps 47.3).  Not under capture nor on a handle that served a request under
 // capture: the two snapshots swap with every request, and a replay reads and writes the one it was
 // captured with.
-// The second snapshot is allocated with a lattice that marches; without memory for it the sums are
-// fused.
+// The second snapshot is allocated with a lattice that marches, if snapshot_pays; without memory for
+// it the sums are fused.
 bool serve_by_snapshot(const fmlbm_handle* h) {
     return h->rho_next && !h->snap_fixed && h->tile_y == kTileYSmall && resolved_variant(h) == FMLBM_VARIANT_PLAIN;
 }
@@ -538,6 +538,16 @@ bool marches(int nc, const fmlbm_lattice& L) {
     }
 }
 
+// Whether requests are served by snapshot and reduction rather than by sums fused into tile steps.  On
+// lattices so wide that a march fills about half of its waves the reduction costs more than the march
+// gains (us per monitored step, fused / snapshot, by fill: binary FP32 36000 x 40 0.48 64.0 / 78.2,
+// 40000 x 32 0.52 58.4 / 65.7, ternary FP32 65536 x 16 0.51 80.8 / 86.6).  Above, neither is far ahead:
+// binary FP32 43000 x 50 0.59 96.3 / 100.6, 1024 x 512 0.65 23.1 / 24.3, 1024^2 0.78 47.3 / 46.0, ternary
+// FP32 1024 x 512 0.69 38.0 / 34.5.
+bool snapshot_pays(const fmlbm_handle* h) {
+    return march_fill(h->nc, h->lattice.nx, h->lattice.ny, h->sms) >= 0.55;
+}
+
 // Device bytes a handle takes where it can get them: the split step's planes, the second density
 // snapshot of a marching lattice.
 size_t scratch_bytes(int nc, const fmlbm_lattice& L) {
@@ -642,12 +652,12 @@ fmlbm_status create_handle(const fmlbm_mixture* mixture, const fmlbm_lattice* la
     }
     cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
     // without memory for these the lattice steps fused, and requests are served by fused sums
-    if (const size_t bytes = scratch_bytes(h->nc, *lattice)) {
-        void** p = marches(h->nc, *lattice) ? &h->rho_next : &h->fields;
-        if (cudaMalloc(p, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            *p = nullptr;
-        }
+    const size_t bytes = scratch_bytes(h->nc, *lattice);
+    const bool snapshot = marches(h->nc, *lattice);
+    void** p = snapshot ? &h->rho_next : &h->fields;
+    if (bytes > 0 && (!snapshot || snapshot_pays(h)) && cudaMalloc(p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        *p = nullptr;
     }
     setup_tma(h);
     *out = h;

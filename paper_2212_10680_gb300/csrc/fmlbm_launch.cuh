@@ -200,12 +200,12 @@ cudaError_t launch_pack(const StepArgs& A, cudaStream_t s) {
 // The marching step: 16 (two components) or 12 (three) warps per multiprocessor.
 template <int NC, int ST, bool SPEC, bool NOALLOC>
 cudaError_t launch_march_as(const StepArgs& A, cudaStream_t s) {
-    constexpr int MINB = NC == 2 ? 4 : 3;
+    constexpr int MINB = march_blocks(NC);
     auto k = march_step<NC, ST, SPEC, NOALLOC, MINB>;
     constexpr size_t smem = march_smem_bytes<NC>();
     FMLBM_ENSURE_SMEM(k, smem);
     const int strips = (A.nx + kMarchCols - 1) / kMarchCols;
-    const int chunk = march_chunk_rows(A.ny, strips, A.sms * MINB * kMarchWarps);
+    const int chunk = march_chunk_rows(A.ny, strips, march_capacity(NC, A.sms));
     const int warps = strips * ((A.ny + chunk - 1) / chunk);
     const Planes P = make_planes(A, NC, kDev16<ST>, ST == ST_F32 ? 4 : 2);
     return launch_kernel(k, dim3((warps + kMarchWarps - 1) / kMarchWarps), dim3(32 * kMarchWarps), smem, s, A.pdl != 0, A,

@@ -67,6 +67,18 @@ inline int march_chunk_rows(int ny, int strips, int capacity) {
 }
 
 constexpr int kMarchWarps = 4;  // warps (neighbouring strips) per block
+// Blocks per multiprocessor, and the warps of one wave.
+constexpr int march_blocks(int nc) { return nc == 2 ? 4 : 3; }
+inline int march_capacity(int nc, int sms) { return sms * march_blocks(nc) * kMarchWarps; }
+// The share of its waves' row iterations that a march spends on the rows it owns: the rest are the
+// four halo rows of a chunk and empty places in the last wave.
+inline double march_fill(int nc, int nx, int ny, int sms) {
+    const int strips = (nx + kMarchCols - 1) / kMarchCols, capacity = march_capacity(nc, sms);
+    const int chunk = march_chunk_rows(ny, strips, capacity);
+    const long long warps = (long long)strips * ((ny + chunk - 1) / chunk);
+    const long long waves = (warps + capacity - 1) / capacity;
+    return (double)strips * ny / ((double)waves * capacity * (chunk + 4));
+}
 
 // Words a lane parks per row: the pulled values (their sums are formed again at the collision:
 // what a block parks is taken from the L1, whose size the step feels).
