@@ -393,7 +393,8 @@ void fmlbm_destroy(fmlbm_handle* h);
 /* ------------------------------------------------------------------------------------
  * Batches: many independent lattices of one component count and storage precision
  * (any sizes, any mixtures) in slots, advanced together by one kernel per time step
- * (two components in float or 16-bit storage on 8-row tiles: one per 48 lattices).  Each lattice's arithmetic is that of a single-lattice plain step, so its
+ * (two components in float or 16-bit storage on 8-row tiles, unless the lattices are many and
+ * small: one per 48 lattices).  Each lattice's arithmetic is that of a single-lattice plain step, so its
  * results are bit-identical to fmlbm_step on its own handle, whatever else shares the
  * batch.  fmlbm_batch_run enqueues chunks of steps, checks every lattice's residual
  * after each chunk and retires it once converged.  Batches are not

@@ -42,9 +42,8 @@ struct Slot {
 
 // The parameters of one launch of the packed batch step.
 struct PackGroup {
-    int n = 0, blocks = 0;
-    int first[kBatchGroup] = {};
-    PackLattice lat[kBatchGroup];
+    int blocks = 0;
+    PackBatch<kBatchGroup> B{};
 };
 
 struct fmlbm_batch {
@@ -109,20 +108,20 @@ cudaError_t launch_batch_step_t(const fmlbm_batch* b, int ahead, bool pdl) {
 }
 template <int ST, bool SPEC, int MAXL>
 cudaError_t launch_batch_pack_as(const fmlbm_batch* b, const PackGroup& G, bool pdl) {
-    PackBatch<MAXL> B;
-    B.n = G.n;
-    std::memcpy(B.first, G.first, sizeof B.first);
-    std::memcpy(B.lat, G.lat, (size_t)G.n * sizeof(PackLattice));
     constexpr size_t smem = sizeof(PackSmem<2, kTileYSmall>);
     auto k = batch_pack<ST, SPEC, MAXL>;
     FMLBM_ENSURE_SMEM(k, smem);
     FMLBM_ENSURE_CARVEOUT(k, 35);  // as the packed step of a single lattice
-    return launch_kernel(k, dim3(G.blocks), dim3(kTX, kTileYSmall), smem, b->stream, pdl, B);
+    // the parameters of fewer lattices are the first bytes of those of more
+    static_assert(offsetof(PackBatch<MAXL>, lat) == offsetof(PackBatch<kBatchGroup>, lat) &&
+                      sizeof(PackBatch<MAXL>) <= sizeof(PackBatch<kBatchGroup>),
+                  "PackBatch<MAXL> is a prefix");
+    return launch_kernel_at(k, dim3(G.blocks), dim3(kTX, kTileYSmall), smem, b->stream, pdl, &G.B);
 }
 template <int ST, bool SPEC>
 cudaError_t launch_batch_pack(const fmlbm_batch* b, int ahead, bool pdl) {
     for (const PackGroup& G : b->groups[(b->since + ahead) & 1]) {
-        const cudaError_t e = G.n <= kBatchGroupSmall ? launch_batch_pack_as<ST, SPEC, kBatchGroupSmall>(b, G, pdl)
+        const cudaError_t e = G.B.n <= kBatchGroupSmall ? launch_batch_pack_as<ST, SPEC, kBatchGroupSmall>(b, G, pdl)
                                                       : launch_batch_pack_as<ST, SPEC, kBatchGroup>(b, G, pdl);
         if (e != cudaSuccess) return e;
         pdl = true;
@@ -130,36 +129,57 @@ cudaError_t launch_batch_pack(const fmlbm_batch* b, int ahead, bool pdl) {
     return cudaSuccess;
 }
 
-// Two components in float or 16-bit storage: the packed step (1000 steps of 16 binaries of 88 to 484
-// nodes a side, FP32, with their creation and read-back: 62.8 ms by the persistent kernel, 46.5 packed).
-bool packed(const fmlbm_batch* b) { return b->nc == 2 && b->precision != FMLBM_FP64 && b->tile_y == kTileYSmall; }
+// Whether the packed step exists for this batch: two components in float or 16-bit storage (1000
+// steps of 16 binaries of 88 to 484 nodes a side, FP32, with their creation and read-back: 62.8 ms by
+// the persistent kernel, 46.5 packed).
+bool packed(const fmlbm_batch* b) {
+    return b->nc == 2 && b->precision != FMLBM_FP64 && b->tile_y == kTileYSmall && !b->captured;
+}
+// Whether the packed step is the faster one for a call of n steps.  Up to 48 lattices are one launch; more
+// are several, each behind the whole of the one before, and pay their start and tail unless each has
+// blocks for more than a wave of the chip's places.  A call of a single step also waits for its
+// launch's parameters (27 KB above 16 lattices) to be copied.  us per step, FP32, persistent kernel ->
+// packed, of a call of 200 steps and of one step that is waited for:
+//   one launch        16 x 32^2  4.6 -> 3.6, 16.7 -> 17.2;  48 x 32^2 (192 blocks) 5.6 -> 4.8, 18.9 -> 19.6;
+//                     24 x 64^2 (384) 6.9 -> 5.9, 19.3 -> 21.9;  48 x 64^2 (768) 11.2 -> 9.1, 23.5 -> 23.7;
+//                     48 x 80^2 (1440) 17.3 -> 13.6, 30.1 -> 28.8
+//   blocks a launch   1024 x 16^2 (93) 23.7 -> 77.5, 37 -> 93;  256 x 32^2 (171) 14.8 -> 27.0, 27 -> 43;
+//                     256 x 64^2 (683) 51.7 -> 62.8, 64 -> 77;  192 x 64^2 (768) 39.6 -> 44.3, 52 -> 58;
+//                     96 x 64^2 (768) 19.2 -> 18.0, 32.4 -> 33.8;  64 x 80^2 (960) 23.1 -> 20.9, 36.1 -> 36.4;
+//                     97 x 96^2 (1164) 44.8 -> 44.6, 58.5 -> 59.4;  256 x 80^2 (1280) 91.5 -> 88.1, 104.6 -> 103.4
+bool pack_pays(const fmlbm_batch* b, long long n) {
+    if (!packed(b)) return false;
+    const size_t launches = b->groups[0].size(), places = (size_t)kBatchPackBlocks * b->sms;
+    if (launches == 1) return n > 1 || b->groups[0][0].B.n <= kBatchGroupSmall || (size_t)b->nwork >= places;
+    return b->nwork >= (n > 1 ? 1.2 : 1.6) * places * launches;
+}
 
 template <int ST, int NC>
-cudaError_t launch_batch_step_nc(const fmlbm_batch* b, int ahead, bool pdl) {
+cudaError_t launch_batch_step_nc(const fmlbm_batch* b, int ahead, bool pdl, bool pack) {
     if (b->tile_y == kTileYLarge) return launch_batch_step_t<ST, NC, kTileYLarge>(b, ahead, pdl);
     if constexpr (NC == 2 && kSpecStep<ST>) {
-        if (!b->captured) return b->spec ? launch_batch_pack<ST, true>(b, ahead, pdl) : launch_batch_pack<ST, false>(b, ahead, pdl);
+        if (pack) return b->spec ? launch_batch_pack<ST, true>(b, ahead, pdl) : launch_batch_pack<ST, false>(b, ahead, pdl);
     }
     return launch_batch_step_t<ST, NC, kTileYSmall>(b, ahead, pdl);
 }
 
 template <int ST>
-cudaError_t launch_batch_step_st(const fmlbm_batch* b, int ahead, bool pdl) {
+cudaError_t launch_batch_step_st(const fmlbm_batch* b, int ahead, bool pdl, bool pack) {
     switch (b->nc) {
-        case 1: return launch_batch_step_nc<ST, 1>(b, ahead, pdl);
-        case 2: return launch_batch_step_nc<ST, 2>(b, ahead, pdl);
-        case 3: return launch_batch_step_nc<ST, 3>(b, ahead, pdl);
-        case 4: return launch_batch_step_nc<ST, 4>(b, ahead, pdl);
+        case 1: return launch_batch_step_nc<ST, 1>(b, ahead, pdl, pack);
+        case 2: return launch_batch_step_nc<ST, 2>(b, ahead, pdl, pack);
+        case 3: return launch_batch_step_nc<ST, 3>(b, ahead, pdl, pack);
+        case 4: return launch_batch_step_nc<ST, 4>(b, ahead, pdl, pack);
     }
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_batch_step(const fmlbm_batch* b, int ahead, bool pdl) {
+cudaError_t launch_batch_step(const fmlbm_batch* b, int ahead, bool pdl, bool pack) {
     switch (b->precision) {
-        case FMLBM_FP64: return launch_batch_step_st<ST_F64>(b, ahead, pdl);
-        case FMLBM_FP32: return launch_batch_step_st<ST_F32>(b, ahead, pdl);
-        case FMLBM_FP16DEV: return launch_batch_step_st<ST_F16DEV>(b, ahead, pdl);
-        default: return launch_batch_step_st<ST_BF16DEV>(b, ahead, pdl);
+        case FMLBM_FP64: return launch_batch_step_st<ST_F64>(b, ahead, pdl, pack);
+        case FMLBM_FP32: return launch_batch_step_st<ST_F32>(b, ahead, pdl, pack);
+        case FMLBM_FP16DEV: return launch_batch_step_st<ST_F16DEV>(b, ahead, pdl, pack);
+        default: return launch_batch_step_st<ST_BF16DEV>(b, ahead, pdl, pack);
     }
 }
 
@@ -229,15 +249,15 @@ void fill_groups(fmlbm_batch* b) {
     for (int p = 0; p < 2; ++p) {
         std::vector<PackGroup>& gs = b->groups[p];
         gs.clear();
-        if (!packed(b) || b->captured) continue;
+        if (!packed(b)) continue;
         for (int k = 0; k < b->capacity; ++k) {
             const Slot& s = b->slots[k];
             if (!s.used || !s.active) continue;
-            if (gs.empty() || gs.back().n == kBatchGroup) gs.emplace_back();
+            if (gs.empty() || gs.back().B.n == kBatchGroup) gs.emplace_back();
             const StepArgs& A = b->h_lat[k].args[(s.steps + p) & 1];
             const Planes P = make_planes(A, 2, dev16, dev16 ? 2 : 4);
             PackGroup& G = gs.back();
-            PackLattice& d = G.lat[G.n];
+            PackLattice& d = G.B.lat[G.B.n];
             d.nx = A.nx;
             d.ny = A.ny;
             d.stencil = A.stencil;
@@ -250,7 +270,7 @@ void fill_groups(fmlbm_batch* b) {
             std::copy(P.g0in, P.g0in + 2, d.g0in);
             std::copy(P.g0out, P.g0out + 2, d.g0out);
             d.mixf = A.mixf;
-            G.first[G.n++] = G.blocks;
+            G.B.first[G.B.n++] = G.blocks;
             G.blocks += b->h_lat[k].nitems;
         }
     }
@@ -328,10 +348,11 @@ fmlbm_status enqueue_steps(fmlbm_batch* b, long long n) {
     BCUDA(b, cudaStreamIsCapturing(b->stream, &cap));
     const bool capturing = cap != cudaStreamCaptureStatusNone;
     b->captured = b->captured || capturing;
+    const bool pack = pack_pays(b, n);
     const int nb = (b->capacity + 127) / 128;
     for (long long done = 0; done < n;) {
         const int m = (int)std::min<long long>(n - done, 1 << 20);
-        for (int k = 0; k < m; ++k) BCUDA(b, launch_batch_step(b, k, k > 0 && !capturing));
+        for (int k = 0; k < m; ++k) BCUDA(b, launch_batch_step(b, k, k > 0 && !capturing, pack));
         b->since += m;
         batch_advance<<<nb, 128, 0, b->stream>>>(b->d_lat, b->capacity, m);
         BCUDA(b, cudaGetLastError());

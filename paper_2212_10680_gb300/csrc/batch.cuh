@@ -91,6 +91,7 @@ struct PackLattice {
 __device__ __forceinline__ bool checked_row(const PackLattice&, int) { return true; }
 constexpr int kBatchGroup = 48;       // lattices in one launch (27 KB of parameters)
 constexpr int kBatchGroupSmall = 16;  // fewer lattices take the launch with less to copy
+constexpr int kBatchPackBlocks = 5;   // blocks per multiprocessor
 template <int MAXL>
 struct PackBatch {
     int n;
@@ -98,7 +99,7 @@ struct PackBatch {
     PackLattice lat[MAXL];
 };
 template <int ST, bool SPEC, int MAXL>
-__global__ void __launch_bounds__(kTX * 8, 5) batch_pack(const __grid_constant__ PackBatch<MAXL> B) {
+__global__ void __launch_bounds__(kTX * 8, kBatchPackBlocks) batch_pack(const __grid_constant__ PackBatch<MAXL> B) {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_batch_pack[];
     int l = 0;

@@ -54,19 +54,33 @@ inline cudaError_t ensure_carveout(std::atomic<unsigned long long>& done, const 
 
 // A launch, programmatic behind the stream's preceding launch if pdl (only for kernels that call
 // pdl_wait before they touch memory).
+struct LaunchSetup {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    LaunchSetup(dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl) {
+        cfg.gridDim = grid;
+        cfg.blockDim = block;
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = pdl ? 1 : 0;
+    }
+    LaunchSetup(const LaunchSetup&) = delete;
+};
 template <typename... P, typename... Q>
 cudaError_t launch_kernel(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl, Q&&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k, static_cast<Q&&>(args)...);
+    LaunchSetup L(grid, block, smem, s, pdl);
+    return cudaLaunchKernelEx(&L.cfg, k, static_cast<Q&&>(args)...);
+}
+// The same for one parameter too large to be passed from hand to hand: the driver copies it once, from
+// `arg`.
+template <typename P>
+cudaError_t launch_kernel_at(void (*k)(P), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool pdl, const void* arg) {
+    LaunchSetup L(grid, block, smem, s, pdl);
+    void* args[] = {const_cast<void*>(arg)};
+    return cudaLaunchKernelExC(&L.cfg, reinterpret_cast<const void*>(k), args);
 }
 
 // Tile heights of the fused step (tile width is one warp).  The host picks one per

@@ -30,3 +30,31 @@ def test_monitored_runs_of_wide_lattices(fm, n, precision, shape):
         out.append(tuple(fm.fmlbm_step_diagnostics(lat.h, 3, n)) + lat.distributions())
         lat.close()
     assert all(np.array_equal(u, v) for u, v in zip(*out))
+
+
+@pytest.mark.parametrize("precision,count,shape", [
+    ("fp32", 64, (96, 96)),       # several packed launches of more than a wave each; single steps by the batch kernel
+    ("bf16dev", 130, (33, 17)),   # small lattices in several launches: the batch kernel
+    ("fp32", 17, (40, 33)),       # one launch with the larger parameters; single steps by the batch kernel
+    ("fp16dev", 5, (50, 41))])    # one launch with the smaller ones
+def test_batches_of_many_lattices(fm, precision, count, shape):
+    # calls of one and of several steps in turn, so that packed and unpacked steps follow each other
+    mixd = mixture_dict(n=2, Tr=1.05, kappa_scale=0.5)
+    b = fm.fmlbm_batch_create(2, precision, count)
+    L = fm.make_lattice(*shape, 0.9, precision=precision)
+    rhos = [smooth_state(2, *shape, seed=k) for k in range(count)]
+    slots = [fm.fmlbm_batch_add(b, fm.mixture_from_dict(mixd), L, r) for r in rhos]
+    for n in (1, 3, 1, 2, 1):
+        fm.fmlbm_batch_step(b, n)
+    nx, ny = shape
+    for k in sorted({0, count // 2, count - 1}):
+        g, F = np.empty((2, 9, ny, nx)), np.empty((2, ny, nx))
+        fm.fmlbm_batch_get_distributions(b, slots[k], g, F)
+        lat = fm.Lattice(fm.mixture_from_dict(mixd), nx, ny, 0.9, precision=precision)
+        fm.fmlbm_set_tile_height(lat.h, 16)
+        lat.init(rhos[k])
+        lat.step(8)
+        want = lat.distributions()
+        lat.close()
+        assert np.array_equal(g, want[0]) and np.array_equal(F, want[1]), k
+    fm.fmlbm_batch_destroy(b)
