@@ -448,9 +448,11 @@ fmlbm_status fmlbm_batch_slot_info(fmlbm_batch* b, int32_t slot, int64_t* steps,
 fmlbm_status fmlbm_batch_moments(fmlbm_batch* b, int32_t slot, double* rho, double* u, double* lnf);
 fmlbm_status fmlbm_batch_get_distributions(fmlbm_batch* b, int32_t slot, double* g, double* force);
 /* Autotuner: times steps_per_trial steps of the current active slots for each tile
- * height (8, 16) and grid size (1, 2, 4, 8 blocks per multiprocessor) and keeps the
- * fastest (without it a batch runs 8-row tiles, 4 blocks per multiprocessor).  The trial steps are real steps of the lattices (the tiling does not change
- * results).  Outputs (may be NULL): chosen tile height, blocks, ms per step. */
+ * height (8, 16) and grid size (1, 2, 4, 8 blocks per multiprocessor; where the step's launches
+ * have a block per tile, that one) and keeps the fastest (without it a batch runs 8-row tiles, 4
+ * blocks per multiprocessor or a block per tile).  The trial steps are real steps of the lattices
+ * (the tiling does not change results).  Outputs (may be NULL): chosen tile height, blocks of a
+ * step, ms per step. */
 fmlbm_status fmlbm_batch_autotune(fmlbm_batch* b, int32_t steps_per_trial, int32_t* tile_y, int32_t* blocks,
                                   double* ms_per_step);
 /* Device bytes held by the batch's lattices. */

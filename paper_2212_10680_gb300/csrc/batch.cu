@@ -811,7 +811,8 @@ fmlbm_status fmlbm_batch_autotune(fmlbm_batch* b, int32_t steps_per_trial, int32
     const int tys[2] = {kTileYSmall, kTileYLarge};
     const int mults[4] = {1, 2, 4, 8};
     float best = 1e30f;
-    int best_ty = b->tile_y, best_mult = b->grid_mult;
+    const int given_mult = b->grid_mult;
+    int best_ty = b->tile_y, best_mult = given_mult, best_blocks = given_mult * b->sms;
     cudaEvent_t e0, e1;
     BCUDA(b, cudaEventCreate(&e0));
     BCUDA(b, cudaEventCreate(&e1));
@@ -821,8 +822,11 @@ fmlbm_status fmlbm_batch_autotune(fmlbm_batch* b, int32_t steps_per_trial, int32
         fmlbm_status st = ensure_work(b);
         if (st != FMLBM_OK) return st;
         if (b->nwork == 0) break;
+        // the packed step has one grid, a block per tile: one trial
+        const bool pack = pack_pays(b, steps_per_trial);
         for (int mult : mults) {
-            b->grid_mult = mult;
+            if (pack && mult != mults[0]) break;
+            b->grid_mult = pack ? given_mult : mult;
             // each trial advances the lattices by real steps: the tiling does not change results
             st = enqueue_steps(b, 1);
             if (st != FMLBM_OK) return st;
@@ -836,7 +840,8 @@ fmlbm_status fmlbm_batch_autotune(fmlbm_batch* b, int32_t steps_per_trial, int32
             if (ms < best) {
                 best = ms;
                 best_ty = ty;
-                best_mult = mult;
+                best_mult = b->grid_mult;
+                best_blocks = pack ? b->nwork : mult * b->sms;
             }
         }
     }
@@ -846,7 +851,7 @@ fmlbm_status fmlbm_batch_autotune(fmlbm_batch* b, int32_t steps_per_trial, int32
     b->grid_mult = best_mult;
     b->work_dirty = true;
     if (tile_y_out) *tile_y_out = best_ty;
-    if (blocks_out) *blocks_out = best_mult * b->sms;
+    if (blocks_out) *blocks_out = best_blocks;
     if (ms_per_step_out) *ms_per_step_out = best / steps_per_trial;
     return FMLBM_OK;
 }

@@ -58,3 +58,17 @@ def test_batches_of_many_lattices(fm, precision, count, shape):
         lat.close()
         assert np.array_equal(g, want[0]) and np.array_equal(F, want[1]), k
     fm.fmlbm_batch_destroy(b)
+
+
+@pytest.mark.parametrize("precision,trials", [("fp32", 5), ("fp64", 8)])   # packed on 8-row tiles; never packed
+def test_batch_autotune_tries_each_grid_once(fm, precision, trials):
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    b = fm.fmlbm_batch_create(2, precision, 2)
+    mix = fm.mixture_from_dict(mixture_dict(n=2, Tr=1.05, kappa_scale=0.5))
+    slot = fm.fmlbm_batch_add(b, mix, fm.make_lattice(100, 70, 1.0, precision=precision), smooth_state(2, 100, 70))
+    ty, blocks, _ = fm.fmlbm_batch_autotune(b, 3)
+    assert fm.fmlbm_batch_slot_info(b, slot)[0] == trials * (1 + 3)
+    tiles = 4 * 9   # of 32 x 8 nodes
+    assert blocks == tiles if precision == "fp32" and ty == 8 else blocks in (sms, 2 * sms, 4 * sms, 8 * sms)
+    fm.fmlbm_batch_destroy(b)
