@@ -112,18 +112,21 @@ def measured_peaks() -> dict:
     return dict(hbm_gbs=6800.0, source="fallback")
 
 
-def step_kernel(variant: str, prec: str, n: int, nodes: int, tile_y: int = 0) -> str:
+MARCH_NODES, MARCH_COLS, PACK_NODES = 1 << 19, 28, 1 << 16   # as the library's launchers choose
+
+
+def step_kernel(variant: str, prec: str, n: int, nx: int, ny: int, tile_y: int = 0, standard: bool = False) -> str:
     """The kernel that a step runs (the two-launch forms by their second)."""
     named = {"tma": "fused_step_tma", "tma_tile": "fused_step_tma", "pair": "fused_step_pair", "multi": "fused_steps"}
     if variant in named:
         return named[variant]
-    if tile_y not in (0, 8):
+    if standard or tile_y not in (0, 8):
         return "fused_step"
     if prec == "fp64" or prec.endswith("lnf64"):
         return "collide_fields"
-    if n in (2, 3) and nodes >= 1 << 19:
+    if n in (2, 3) and nx * ny >= MARCH_NODES and 4 * (-(-nx // MARCH_COLS) * MARCH_COLS) <= 5 * nx:
         return "march_step"
-    return "pack_step" if n == 2 and nodes >= 1 << 16 else "fused_step"
+    return "pack_step" if n == 2 and nx * ny >= PACK_NODES else "fused_step"
 
 
 def profile_traffic(kernel: str, workload_key: str, precision: str):
@@ -485,7 +488,7 @@ def ternary_forms(fmlbm, torch, stream, dev, steps, warmup, flush):
         out[prec] = dict(value=r["n"] * r["nodes"] / per / 1e9, unit="component-GLUPS", ms_per_step=1e3 * per,
                          steps=k, roofline=dict(bound="hbm", achieved=achieved, peak=peak["hbm_gbs"], unit="GB/s",
                                                 frac=achieved / peak["hbm_gbs"],
-                                                traffic=profile_traffic(step_kernel("plain", prec, r["n"], r["nodes"]),
+                                                traffic=profile_traffic(step_kernel("plain", prec, r["n"], w["nx"], w["ny"]),
                                                                         "ternary4096", prec),
                                                 algorithmic_bytes_per_component_node=ALGO_BYTES[prec]),
                          clocks=r["clocks"])
@@ -545,7 +548,7 @@ def run_ours(args, w, rank, world, dist):
     algo = ALGO_BYTES[prec] * n * nodes
     peak = measured_peaks()
     achieved = algo / per_launch_s / 1e9
-    kernel_name = step_kernel(variant, prec, n, nodes, tuned["tile_y"] if tuned else args.tile_y)
+    kernel_name = step_kernel(variant, prec, n, nx, ny, tuned["tile_y"] if tuned else args.tile_y)
     # the committed counters describe the workload at its own size only
     traffic = None if args.size else profile_traffic(kernel_name, args.workload, prec)
     e2e = _e2e_rate(fmlbm, torch, w, prec, args.steps, stream, dev, dist)
