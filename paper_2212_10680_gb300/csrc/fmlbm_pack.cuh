@@ -16,14 +16,11 @@ constexpr size_t kPackNodes = 1 << 16;
 // A field of the tile with a halo of H nodes, pairs of components side by side.
 template <int NC, int TY, int H>
 struct PackTile {
-    static constexpr int W = kTX + 2 * H, R = TY + 2 * H;
-    float2 p[NC >= 2 ? NC / 2 : 1][NC >= 2 ? R : 1][NC >= 2 ? W : 1];
-    float s[(NC & 1) ? R : 1][(NC & 1) ? W : 1];
+    static_assert(NC % 2 == 0, "components come in pairs");
+    float2 p[NC / 2][TY + 2 * H][kTX + 2 * H];
 };
 template <int NC, int TY, int H>
 __device__ __forceinline__ float2* tile_row(PackTile<NC, TY, H>& t, PairOf of, int cy) { return t.p[of.k][cy]; }
-template <int NC, int TY, int H, int I>
-__device__ __forceinline__ float* tile_row(PackTile<NC, TY, H>& t, LastOf<I>, int cy) { return t.s[cy]; }
 
 template <int NC, int TY>
 struct PackSmem {
@@ -35,8 +32,9 @@ struct PackSmem {
 
 // Finite differences at column cx of three consecutive rows (n above, c, s below): the
 // operations of grad_at and lap_at.
-template <typename V>
-__device__ __forceinline__ void grad_tile(const V* rn, const V* rc, const V* rs, int cx, int stencil, V& gx, V& gy) {
+__device__ __forceinline__ void grad_tile(const float2* rn, const float2* rc, const float2* rs, int cx, int stencil,
+                                          float2& gx, float2& gy) {
+    using V = float2;
     const V e = rc[cx + 1], w = rc[cx - 1], n = rn[cx], s = rs[cx];
     if (stencil == 1) {
         gx = vmul(vbc<V>(0.5f), vsub(e, w));
@@ -48,8 +46,8 @@ __device__ __forceinline__ void grad_tile(const V* rn, const V* rc, const V* rs,
         gy = vfma(vsub(n, s), third, vmul(vsub(vadd(ne, nw), vadd(sw, se)), twelfth));
     }
 }
-template <typename V>
-__device__ __forceinline__ V lap_tile(const V* rn, const V* rc, const V* rs, int cx, int stencil) {
+__device__ __forceinline__ float2 lap_tile(const float2* rn, const float2* rc, const float2* rs, int cx, int stencil) {
+    using V = float2;
     const V c = rc[cx];
     const V ax = vadd(vadd(rc[cx + 1], rc[cx - 1]), vadd(rn[cx], rs[cx]));
     const V m4 = vbc<V>(-4.f);
@@ -66,11 +64,10 @@ __device__ __forceinline__ void pack_phi(const MixConstT<float>& m, PackSmem<NC,
         of(L) = lap_tile(tile_row(S.rt, of, cy + 2), tile_row(S.rt, of, cy + 1), tile_row(S.rt, of, cy), cx + 1, stencil);
     });
     each_group<NC>([&](auto of) {
-        using V = typename decltype(of)::V;
-        V Gi = vmul(of.col(m.kap, 0), vbc<V>(comp(L, 0)));
+        float2 Gi = vmul(of.col(m.kap, 0), vbc<float2>(comp(L, 0)));
 #pragma unroll
-        for (int j = 1; j < NC; ++j) Gi = vfma(of.col(m.kap, j), vbc<V>(comp(L, j)), Gi);
-        tile_row(S.G, of, cy)[cx] = vfma(vbc<V>(-m.RT), tile_row(S.lf, of, cy)[cx], Gi);
+        for (int j = 1; j < NC; ++j) Gi = vfma(of.col(m.kap, j), vbc<float2>(comp(L, j)), Gi);
+        tile_row(S.G, of, cy)[cx] = vfma(vbc<float2>(-m.RT), tile_row(S.lf, of, cy)[cx], Gi);
     });
 }
 
@@ -97,8 +94,7 @@ __device__ __forceinline__ void pack_pull(const PL& P, bool inner, int wx, int w
 template <int NC>
 __device__ __forceinline__ void pack_rho(const MixConstT<float>& m, const Comps<NC> (&g)[9], Comps<NC>& r, Comps<NC>& rt) {
     each_group<NC>([&](auto of) {
-        using V = typename decltype(of)::V;
-        V s = of(g[0]);
+        float2 s = of(g[0]);
 #pragma unroll
         for (int a = 1; a < 9; ++a) s = vadd(s, of(g[a]));
         of(r) = s;
@@ -137,7 +133,6 @@ __device__ __forceinline__ void pack_tile(const AT& A, const PL& P, PackSmem<NC,
         constexpr bool inner = decltype(inner_c)::value;
         constexpr int RING = 4 * (kTX + 4) + 4 * TY;
         static_assert(RING <= NT, "one ring node per thread");
-        constexpr bool RING_FIRST = !(ST == ST_F32 && NC >= 3);
         const bool has_ring = tid < RING;
         int bx = 0, by = 0;
         Comps<NC> rrt;
@@ -157,24 +152,20 @@ __device__ __forceinline__ void pack_tile(const AT& A, const PL& P, PackSmem<NC,
                 each_group<NC>([&](auto of) { tile_row(S.lf, of, by - 1)[bx - 1] = of(lnf); });
             }
         };
-        if (RING_FIRST && has_ring) pull_ring();
+        if (has_ring) pull_ring();
         pack_pull<NC, ST>(P, inner, inner ? x : wrap(x, nx), inner ? y : wrap(y, ny), nx, ny, g);
-        if (RING_FIRST && has_ring) put_ring();
+        if (has_ring) put_ring();
         Comps<NC> rt, lnf;
         pack_rho<NC>(m, g, r, rt);
         each_group<NC>([&](auto of) {
-            using V = typename decltype(of)::V;
-            constexpr bool PAIR = std::is_same<V, float2>::value;
-            int i0 = NC - 1;
-            if constexpr (PAIR) i0 = 2 * of.k;
-            V h[9], jxi, jyi;
+            float2 h[9], jxi, jyi;
 #pragma unroll
             for (int a = 0; a < 9; ++a) h[a] = of(g[a]);
             moment_j(h, true, jxi, jyi);
 #pragma unroll
-            for (int l = 0; l < (PAIR ? 2 : 1); ++l) {
-                jx = i0 + l == 0 ? lane(jxi, l) : vadd(jx, lane(jxi, l));
-                jy = i0 + l == 0 ? lane(jyi, l) : vadd(jy, lane(jyi, l));
+            for (int l = 0; l < 2; ++l) {
+                jx = 2 * of.k + l == 0 ? lane(jxi, l) : vadd(jx, lane(jxi, l));
+                jy = 2 * of.k + l == 0 ? lane(jyi, l) : vadd(jy, lane(jyi, l));
             }
             tile_row(S.rt, of, ty + 2)[tx + 2] = of(rt);
         });
@@ -196,10 +187,6 @@ __device__ __forceinline__ void pack_tile(const AT& A, const PL& P, PackSmem<NC,
             }
             domain_check<NC, float>(A, rr, ll, beta, x, 0, y, 1u);
         }
-        if (!RING_FIRST && has_ring) {
-            pull_ring();
-            put_ring();
-        }
     };
     // no periodic wrap anywhere in this block's reach (tile + 2 halo + 1 pull)
     if (x0 >= 3 && x0 + kTX + 3 <= nx && y0 >= 3 && y0 + TY + 3 <= ny) phase1(std::true_type());
@@ -220,38 +207,31 @@ __device__ __forceinline__ void pack_tile(const AT& A, const PL& P, PackSmem<NC,
         float Ftx = 0.f, Fty = 0.f, ux = 0.f, uy = 0.f;
         Comps<NC> Fx, Fy, grx, gry;
         auto force = [&](auto of) {
-            using V = typename decltype(of)::V;
-            constexpr bool PAIR = std::is_same<V, float2>::value;
-            int i0 = NC - 1;
-            if constexpr (PAIR) i0 = 2 * of.k;
-            V px, py, rx, ry;
-            grad_tile<V>(tile_row(S.G, of, ty + 2), tile_row(S.G, of, ty + 1), tile_row(S.G, of, ty), tx + 1, stencil, px, py);
-            grad_tile<V>(tile_row(S.rt, of, ty + 3), tile_row(S.rt, of, ty + 2), tile_row(S.rt, of, ty + 1), tx + 2, stencil,
-                         rx, ry);
-            const V rti = tile_row(S.rt, of, ty + 2)[tx + 2];
+            float2 px, py, rx, ry;
+            grad_tile(tile_row(S.G, of, ty + 2), tile_row(S.G, of, ty + 1), tile_row(S.G, of, ty), tx + 1, stencil, px, py);
+            grad_tile(tile_row(S.rt, of, ty + 3), tile_row(S.rt, of, ty + 2), tile_row(S.rt, of, ty + 1), tx + 2, stencil, rx,
+                      ry);
+            const float2 rti = tile_row(S.rt, of, ty + 2)[tx + 2];
             of(grx) = vmul(rx, of.of(m.M));
             of(gry) = vmul(ry, of.of(m.M));
             of(Fx) = vmul(rti, px);
             of(Fy) = vmul(rti, py);
 #pragma unroll
-            for (int l = 0; l < (PAIR ? 2 : 1); ++l) {
-                Ftx = i0 + l == 0 ? lane(of(Fx), l) : vadd(Ftx, lane(of(Fx), l));
-                Fty = i0 + l == 0 ? lane(of(Fy), l) : vadd(Fty, lane(of(Fy), l));
+            for (int l = 0; l < 2; ++l) {
+                Ftx = 2 * of.k + l == 0 ? lane(of(Fx), l) : vadd(Ftx, lane(of(Fx), l));
+                Fty = 2 * of.k + l == 0 ? lane(of(Fy), l) : vadd(Fty, lane(of(Fy), l));
             }
         };
         auto collide = [&](auto of) {
-            using V = typename decltype(of)::V;
-            constexpr bool PAIR = std::is_same<V, float2>::value;
-            int i0 = NC - 1;
-            if constexpr (PAIR) i0 = 2 * of.k;
-            V h[9];
+            float2 h[9];
 #pragma unroll
             for (int a = 0; a < 9; ++a) h[a] = of(g[a]);
-            collide_node<false, V, float>(m, h, of(r), vbc<V>(ux), vbc<V>(uy), of(Fx), of(Fy), of(grx), of(gry),
-                                          [&](int a, V v) {
+            collide_node<false, float2, float>(m, h, of(r), vbc<float2>(ux), vbc<float2>(uy), of(Fx), of(Fy), of(grx), of(gry),
+                                               [&](int a, float2 v) {
 #pragma unroll
-                                              for (int l = 0; l < (PAIR ? 2 : 1); ++l) store_gp<ST>(P, i0 + l, a, node, lane(v, l));
-                                          });
+                                                   for (int l = 0; l < 2; ++l)
+                                                       store_gp<ST>(P, 2 * of.k + l, a, node, lane(v, l));
+                                               });
         };
         if (lagged) {
             asm volatile("cp.async.wait_all;\n" ::: "memory");

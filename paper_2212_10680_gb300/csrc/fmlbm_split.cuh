@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kTX* TY) collide_fields(const __grid_constant_
     prefetch_force<Real, NC, TY>(A, S, tx, ty, x, y);
     const Real* f = static_cast<const Real*>(A.fields);
     // rho~ on the tile + 2 and ln f on the tile + 1
-    constexpr int W2 = kTX + 4, W1 = kTX + 2;
+    constexpr int W2 = kTX + 4;
     for (int e = tid; e < W2 * (TY + 4); e += kTX * TY) {
         const int by = e / W2, bx = e - by * W2;
         const size_t node = (size_t)wrap(y0 - 2 + by, ny) * nx + wrap(x0 - 2 + bx, nx);
@@ -102,7 +102,6 @@ __global__ void __launch_bounds__(kTX* TY) collide_fields(const __grid_constant_
             if (in) S.lf.v[i][by - 1][bx - 1] = f[(size_t)(NC + i) * nxy + node];
         }
     }
-    static_assert(W1 == kTX + 2, "ln f box inside the rho~ box");
     Real g[NC][9], r[NC], jx = Real(0), jy = Real(0);
     if (valid) {
         const int xm = x == 0 ? nx - 1 : x - 1, xp = x == nx - 1 ? 0 : x + 1;
