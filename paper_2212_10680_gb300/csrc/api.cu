@@ -43,6 +43,7 @@ struct fmlbm_handle {
     float* g0[2] = {nullptr, nullptr};  // DEV: float planes a = 0
     void* F[2] = {nullptr, nullptr};
     int cur = 0;
+    void* snapshots = nullptr;    // the allocation of the density snapshots
     void* rho_prev = nullptr;     // storage arithmetic type
     int have_prev = 0;
     void* rho_next = nullptr;        // a second snapshot, for marching steps that write the densities they read
@@ -420,8 +421,7 @@ void release(fmlbm_handle* h) {
         if (h->g0[k]) cudaFree(h->g0[k]);
         if (h->F[k]) cudaFree(h->F[k]);
     }
-    if (h->rho_prev) cudaFree(h->rho_prev);
-    if (h->rho_next) cudaFree(h->rho_next);
+    if (h->snapshots) cudaFree(h->snapshots);
     if (h->partial) cudaFree(h->partial);
     if (h->done) cudaFree(h->done);
     if (h->fields) cudaFree(h->fields);
@@ -548,15 +548,13 @@ bool snapshot_pays(const fmlbm_handle* h) {
     return march_fill(h->nc, h->lattice.nx, h->lattice.ny, h->sms) >= 0.55;
 }
 
-// Device bytes a handle takes where it can get them: the split step's planes, the second density
-// snapshot of a marching lattice.
-size_t scratch_bytes(int nc, const fmlbm_lattice& L) {
-    const size_t nxy = (size_t)L.nx * (size_t)L.ny;
+// Device bytes of the split step's scratch planes (0: the lattice does not take it).
+size_t fields_bytes(int nc, const fmlbm_lattice& L) {
     const bool f64 = L.precision == FMLBM_FP64;
-    if ((f64 || L.precision == FMLBM_FP16DEV_LNF64 || L.precision == FMLBM_BF16DEV_LNF64) &&
-        L.formulation == FMLBM_WELL_BALANCED)
-        return split_planes(nc, f64) * nxy * real_size(L.precision);
-    return marches(nc, L) ? nc * nxy * sizeof(float) : 0;
+    if ((!f64 && L.precision != FMLBM_FP16DEV_LNF64 && L.precision != FMLBM_BF16DEV_LNF64) ||
+        L.formulation != FMLBM_WELL_BALANCED)
+        return 0;
+    return split_planes(nc, f64) * (size_t)L.nx * (size_t)L.ny * real_size(L.precision);
 }
 
 // Byte ranges [p, p + bytes) that must not overlap (null entries are skipped).
@@ -621,7 +619,16 @@ fmlbm_status create_handle(const fmlbm_mixture* mixture, const fmlbm_lattice* la
         if (g0b) ok = ok && cudaMalloc((void**)&h->g0[k], g0b) == cudaSuccess;
         ok = ok && cudaMalloc(&h->F[k], fb) == cudaSuccess;
     }
-    ok = ok && cudaMalloc(&h->rho_prev, (size_t)h->nc * nxy * real_size(lattice->precision)) == cudaSuccess;
+    // a marching lattice's two density snapshots in one allocation (by a second one creating a 1024^2
+    // binary took 372 us instead of 306); without memory for both, one
+    const size_t rb = ((size_t)h->nc * nxy * real_size(lattice->precision) + 255) / 256 * 256;
+    cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
+    if (ok && marches(h->nc, *lattice) && snapshot_pays(h)) {
+        if (cudaMalloc(&h->snapshots, 2 * rb) == cudaSuccess) h->rho_next = static_cast<char*>(h->snapshots) + rb;
+        else cudaGetLastError();
+    }
+    ok = ok && (h->snapshots || cudaMalloc(&h->snapshots, rb) == cudaSuccess);
+    h->rho_prev = h->snapshots;
     ok = ok && cudaMalloc(&h->partial, kDiagSlots * (size_t)reduce_blocks(lattice->nx, lattice->ny) * (kMaxC + 2) *
                                            sizeof(double)) == cudaSuccess;
     ok = ok && cudaMalloc((void**)&h->diag_dev, (kDiagSlots * kDiagWords + 2) * sizeof(double)) == cudaSuccess;
@@ -650,14 +657,11 @@ fmlbm_status create_handle(const fmlbm_mixture* mixture, const fmlbm_lattice* la
         delete h;
         return FMLBM_E_CUDA;
     }
-    cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
-    // without memory for these the lattice steps fused, and requests are served by fused sums
-    const size_t bytes = scratch_bytes(h->nc, *lattice);
-    const bool snapshot = marches(h->nc, *lattice);
-    void** p = snapshot ? &h->rho_next : &h->fields;
-    if (bytes > 0 && (!snapshot || snapshot_pays(h)) && cudaMalloc(p, bytes) != cudaSuccess) {
+    // the split step's planes; without them (no memory left) the lattice steps fused
+    const size_t planes = fields_bytes(h->nc, *lattice);
+    if (planes > 0 && cudaMalloc(&h->fields, planes) != cudaSuccess) {
         cudaGetLastError();
-        *p = nullptr;
+        h->fields = nullptr;
     }
     setup_tma(h);
     *out = h;
@@ -729,7 +733,8 @@ const char* fmlbm_last_error(const fmlbm_handle* h) { return h ? h->last_error.c
 
 fmlbm_status fmlbm_lattice_bytes(int32_t n_components, const fmlbm_lattice* lattice, size_t* bytes) {
     if (!lattice || !bytes || n_components < 1 || n_components > FMLBM_MAX_COMPONENTS) return FMLBM_E_INVALID_ARG;
-    *bytes = fmlbm_internal_batched_bytes(n_components, *lattice) + scratch_bytes(n_components, *lattice);
+    *bytes = fmlbm_internal_batched_bytes(n_components, *lattice) + fields_bytes(n_components, *lattice) +
+             (marches(n_components, *lattice) ? (size_t)n_components * lattice->nx * lattice->ny * sizeof(float) : 0);
     return FMLBM_OK;
 }
 
