@@ -3,7 +3,7 @@
 Default workload: the binary PR vapour-liquid system in lattice units, a circular
 liquid droplet of radius 200 in vapour on a periodic 1024 x 1024 D2Q9 lattice, FP32
 storage and arithmetic, isotropic stencils, lagged velocity force, tau = 1.0, seeded
-1% noise.  One "step" is one time step of the whole method (one fused kernel
+1% noise.  One "step" is one time step of the whole method (one kernel
 launch).  Prints ONE JSON line (rank 0).
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
@@ -441,7 +441,7 @@ def _pool_init():
 
 def small_binary_fp64(fmlbm, torch, stream, dev, gpu_steps=2000, oracle_steps=20):
     """The small parity configuration (64 x 64 binary slab, FP64, tau 1): GPU and oracle
-    milliseconds per step on the same lattice (the GPU run is latency-bound: 4,096 nodes)."""
+    milliseconds per step on the same lattice (the GPU run is bound by the FP64 instructions of its 128 warps: 4,096 nodes)."""
     from paper_2212_10680_gb300 import inputs
     wl = json.load(open(os.path.join(ROOT, "tests", "golden", "workloads.json")))["binary"]
     rho = inputs.with_noise(inputs.slab(wl["slab"]["rt_vapour"], wl["slab"]["rt_liquid"], 64, 64, 0.5, 4.0), 0.01, 1)
@@ -471,7 +471,7 @@ def small_binary_fp64(fmlbm, torch, stream, dev, gpu_steps=2000, oracle_steps=20
     oracle_ms = 1e3 * (time.perf_counter() - t0) / oracle_steps
     return dict(workload="binary PR flat slab 64x64, FP64, tau 1, isotropic, lagged", gpu_ms_per_step=gpu_ms,
                 gpu_steps=gpu_steps, oracle_ms_per_step=oracle_ms, oracle_steps=oracle_steps,
-                note="GPU: launch-bound (4,096 nodes per step); oracle: numpy, one thread")
+                note="GPU: bound by FP64 issue (4,096 nodes: 128 warps on 608 sub-partitions); oracle: numpy, one thread")
 
 
 def ternary_forms(fmlbm, torch, stream, dev, steps, warmup, flush):
@@ -587,7 +587,7 @@ def run_ours(args, w, rank, world, dist):
                     l2="flushed between timed steps (256 MB write, then read: clean lines, none of the step's)",
                     e2e="fmlbm_init from pinned host memory, then fmlbm_step_diagnostics: every step's masses, "
                         "residual and error latch copied to the host",
-                    timing="CUDA events around each fused launch on the launching stream",
+                    timing="CUDA events around each step on the launching stream",
                     step_ms_spread=dict(median=statistics.median(ms), min=min(ms), max=max(ms))),
         roofline=dict(bound="hbm", achieved=achieved, peak=peak["hbm_gbs"], unit="GB/s",
                       frac=achieved / peak["hbm_gbs"], traffic=traffic, peak_source=peak["source"],
@@ -635,8 +635,8 @@ SWEEP_FIRST = 20
 
 def run_batch(args, rank, world, dist=None, summary=False):
     """Batched P-x sweep: independent binary lattices (side 4 x U{16..max_side / 4}, feeds z1 swept
-    0.12..0.95 at fixed T), one persistent multi-lattice step per time step, graph-captured
-    chunks, per-lattice retirement; against the same lattices run one after another with
+    0.12..0.95 at fixed T), stepped together in chunks by the batch kernels, with per-lattice
+    retirement; against the same lattices run one after another with
     single-lattice handles and the same retirement rule.  Each lattice starts as Section V.B
     starts an envelope point: the flat interface of Eq. eqInit (W = 4) between the flash phases
     at S_V = 0.5, unperturbed.  A lattice retires when its phase measure (the mean of ln rho_i

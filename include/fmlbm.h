@@ -195,8 +195,8 @@ fmlbm_status fmlbm_init(fmlbm_handle* h, const double* rho_host);
  * the handle's stream before the call's work completes; not retained). */
 fmlbm_status fmlbm_init_device(fmlbm_handle* h, const double* rho_device);
 
-/* Enqueues nsteps (>= 0) full time steps (steps 1-9 of Section III.B, one fused
- * kernel launch per step; one launch for all of them with FMLBM_VARIANT_MULTI) on the
+/* Enqueues nsteps (>= 0) full time steps (steps 1-9 of Section III.B; one kernel launch per
+ * step, two in FP64 and with ln f in FP64, one for all of them with FMLBM_VARIANT_MULTI) on the
  * handle's stream.  Asynchronous: kernel-side errors surface at the next synchronising
  * call. */
 fmlbm_status fmlbm_step(fmlbm_handle* h, int64_t nsteps);
@@ -230,9 +230,10 @@ fmlbm_status fmlbm_diagnostics(fmlbm_handle* h, double* mass, double* residual, 
  * loop).  fmlbm_diagnostics_async asks for the diagnostics above of the current state
  * and returns at once with a ticket (requests repeated before the next step share
  * one).  Nothing is computed yet: the next fmlbm_step computes them inside its first
- * time step, from the distributions that step reads anyway (every step variant), so a
+ * time step, from the distributions that step reads anyway (every step variant; a marching
+ * step writes the densities beside, and a second kernel sums them), so a
  * loop that steps and asks
- * every step adds no extra pass over the lattice; if no step follows,
+ * every step adds no extra pass over the distributions; if no step follows,
  * fmlbm_diagnostics_wait runs the separate reduction.  Results are bit-identical either
  * way.  The final sum and the copies to the host of a request served inside a step run
  * on a second, non-blocking stream of the handle at the highest stream priority, ordered
@@ -281,8 +282,8 @@ fmlbm_status fmlbm_set_state(fmlbm_handle* h, const void* buf, size_t bytes);
 
 /* Tuning: height (8, 16 or 32 rows) of the 32-column tile each thread block of the
  * plain fused step owns (moments always use 8 or 16).  Results do not depend on it
- * (bit-identical).  Default: 8, with which the library takes the fastest form measured on
- * GB300 for the lattice's size, components and storage: 32 x 8 tiles, with two components
+ * (bit-identical).  Default: 8, with which the library takes the form measured fastest on
+ * GB300 over lattice sizes, components and storage: 32 x 8 tiles, with two components
  * per packed value from 2^16 nodes on (two components), warps that march over the rows from
  * 2^19 nodes on (two and three components, float and 16-bit storage; a second density snapshot,
  * for their diagnostics, is allocated with the lattice), or two launches per
@@ -291,8 +292,8 @@ fmlbm_status fmlbm_set_state(fmlbm_handle* h, const void* buf, size_t bytes);
 fmlbm_status fmlbm_set_tile_height(fmlbm_handle* h, int32_t tile_y);
 
 /* Which kernel advances the lattice.  PLAIN: the step with per-thread pulls from global
- * memory, one node per thread (see fmlbm_set_tile_height).  PAIR: the same step with two nodes per thread (32
- * columns apart in a 64-column tile) whose float arithmetic runs as packed two-lane
+ * memory, in the form that the lattice takes (see fmlbm_set_tile_height).  PAIR: the step with two
+ * nodes per thread (32 columns apart in a 64-column tile) whose float arithmetic runs as packed two-lane
  * instructions; float and 16-bit storage, well-balanced formulation, 8-row tiles.  TMA: a persistent fused step whose blocks copy each wrap-free tile of
  * 32 x 8 nodes (every plane plus a 3-node halo) into shared memory with one bulk tensor
  * copy, double-buffered so the next tile's copy overlaps the current tile's arithmetic;
@@ -300,8 +301,8 @@ fmlbm_status fmlbm_set_tile_height(fmlbm_handle* h, int32_t tile_y);
  * tile per block and a single stage, as many blocks per multiprocessor as shared memory
  * admits (the pulled values wait in shared memory).  All give bit-identical results.  The
  * TMA forms are available for FP32 and 16-bit storage with nx a multiple of 4 (FP32) or 8
- * (16-bit) and a lattice of at least 38 x 14.  AUTO (default): PLAIN, which matched or beat
- * the other forms on the workloads measured on GB300; fmlbm_autotune measures the lattice
+ * (16-bit) and a lattice of at least 38 x 14.  AUTO (default): PLAIN, the fastest on the
+ * workloads measured on GB300; fmlbm_autotune measures the lattice
  * at hand instead.  Every form performs the same operations per node, each rounded once,
  * and gives the same bits.  Asking for a form where it is not available returns
  * FMLBM_E_UNSUPPORTED.
@@ -542,7 +543,7 @@ void fmlbm_server_destroy(fmlbm_server* s);
  * the rows of its neighbours its update reads.  The fused step reads distributions up to
  * three rows away from a node (the pulls of the 2-node halo of rho~ of steps 6-7), so each
  * slab holds its own ny / nslabs rows plus three ghost rows above and below (a lattice of
- * ny / nslabs + 6 rows stepped by the ordinary fused step), and after every step the ghost
+ * ny / nslabs + 6 rows stepped by the ordinary step), and after every step the ghost
  * rows of every distribution plane are refreshed from the neighbouring slabs' boundary rows
  * by cudaMemcpy2DAsync copies (the halo exchange; between devices these would be peer
  * copies).  The slabs' own rows then evolve bit for bit as the undivided lattice does.  All

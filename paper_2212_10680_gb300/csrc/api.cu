@@ -312,11 +312,10 @@ cudaError_t dispatch_step_tma(const fmlbm_handle* h, const StepArgs& A, bool sin
     }
 }
 
-// AUTO resolves to the plain step: it matched or beat every other form on the workloads
-// measured on GB300 (1024^2 binary FP32: 39 us per step against 47 us for the paired step;
-// 4096^2 ternary FP32 and BF16 deviations: 1.6x faster than the paired step, which issues
-// 40% fewer instructions per node but keeps fewer warps resident); fmlbm_autotune measures
-// the lattice at hand instead.  Every form gives the same bits.
+// AUTO resolves to the plain step: it was the fastest form on every workload measured on GB300 (us
+// per step, plain / paired / TMA / TMA_TILE / multi-step: 1024^2 binary FP32 31.6 / 45.1 / 54.5 / 46.4 /
+// 51.4, 4096^2 ternary FP32 766 / 1022 / 1127 / 1254 / 1230, BF16 deviations 633 / 939 / 812 / 793 /
+// 1056); fmlbm_autotune measures the lattice at hand instead.  Every form gives the same bits.
 int resolved_variant(const fmlbm_handle* h) {
     if (h->variant == FMLBM_VARIANT_AUTO) return FMLBM_VARIANT_PLAIN;
     return h->variant;

@@ -191,9 +191,11 @@ template <int NC, int ST>
 cudaError_t launch_split(const StepArgs& A, cudaStream_t s) {
     // Two-row blocks spread a small lattice over the multiprocessors; from 2^16 nodes on there are
     // more 8-row blocks than multiprocessors and the smaller halo counts.  us per step, 8 -> 2 rows,
-    // binary FP64: 64^2 29.6 -> 18.3, 128^2 29.8 -> 19.6, 192^2 30.1 -> 31.8, 256^2 54.5 -> 53.7,
-    // 384^2 104 -> 113, 1024^2 672 -> 728; ln f in FP64 over BF16: 64^2 11.2 -> 8.9, 256^2 17.4 -> 17.1,
-    // 384^2 30.8 -> 32.5.
+    // binary FP64: 64^2 29.7 -> 18.2, 128^2 29.8 -> 19.6, 256^2 54.3 -> 54.0, 384^2 104 -> 114, 512^2
+    // 179 -> 194, 1024^2 676 -> 731; ln f in FP64 over BF16: 64^2 11.2 -> 8.8, 256^2 17.3 -> 17.0, 384^2
+    // 31.0 -> 32.5, 512^2 51.7 -> 54.2.  The node count is a rough measure of what decides near the line,
+    // whole waves of blocks: 192^2 (30.0 -> 32.1, 11.5 -> 12.2) and 320 x 256 (79.0 -> 67.8, 24.1 -> 20.6)
+    // are on the slower side of it.
     return (size_t)A.nx * A.ny <= 65536 ? launch_split_ty<NC, ST, 2>(A, s) : launch_split_ty<NC, ST, 8>(A, s);
 }
 

@@ -15,7 +15,8 @@
 // The tile step is bound by its blocks' phases: every block loads, then computes (6,000 of 14,700
 // cycles of a block pass until its loads have come), its instructions (816 per node, binary FP32)
 // are half halo work, and its shared tiles and halo pulls take 71 % of the L1 data pipe.  Here the
-// loads stay in flight, a node takes 500 instructions, and 48 % of the L1 data pipe is used.  The
+// loads stay in flight, a node takes 513 instructions, and 40 % of the L1 data pipe is used; what
+// bounds it is the latency of the loads that 16 warps (12 with three components) keep in flight.  The
 // first and last two columns of a warp are halo (28 of 32 owned), a chunk of H rows pulls H + 4 and
 // evaluates ln f on H + 2.  Deeper prefetch (two rows), parking in registers (168 registers, 31.3 us
 // on the 1024^2 binary), pulling twice instead of parking (38.5), 20 warps per multiprocessor (49)
