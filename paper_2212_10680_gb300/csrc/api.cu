@@ -618,16 +618,6 @@ fmlbm_status create_handle(const fmlbm_mixture* mixture, const fmlbm_lattice* la
         if (g0b) ok = ok && cudaMalloc((void**)&h->g0[k], g0b) == cudaSuccess;
         ok = ok && cudaMalloc(&h->F[k], fb) == cudaSuccess;
     }
-    // a marching lattice's two density snapshots in one allocation (by a second one creating a 1024^2
-    // binary took 372 us instead of 306); without memory for both, one
-    const size_t rb = ((size_t)h->nc * nxy * real_size(lattice->precision) + 255) / 256 * 256;
-    cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
-    if (ok && marches(h->nc, *lattice) && snapshot_pays(h)) {
-        if (cudaMalloc(&h->snapshots, 2 * rb) == cudaSuccess) h->rho_next = static_cast<char*>(h->snapshots) + rb;
-        else cudaGetLastError();
-    }
-    ok = ok && (h->snapshots || cudaMalloc(&h->snapshots, rb) == cudaSuccess);
-    h->rho_prev = h->snapshots;
     ok = ok && cudaMalloc(&h->partial, kDiagSlots * (size_t)reduce_blocks(lattice->nx, lattice->ny) * (kMaxC + 2) *
                                            sizeof(double)) == cudaSuccess;
     ok = ok && cudaMalloc((void**)&h->diag_dev, (kDiagSlots * kDiagWords + 2) * sizeof(double)) == cudaSuccess;
@@ -645,6 +635,17 @@ fmlbm_status create_handle(const fmlbm_mixture* mixture, const fmlbm_lattice* la
     for (int k = 0; k < kDiagSlots; ++k)
         ok = ok && cudaEventCreateWithFlags(&h->diag_ev[k], cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaMallocHost((void**)&h->err_host, sizeof(ErrorLatch)) == cudaSuccess;
+    // last of the device memory a lattice needs, so that a second snapshot takes from none of it: a
+    // marching lattice's two density snapshots in one allocation (by a second one creating a 1024^2
+    // binary took 372 us instead of 306); without memory for both, one
+    const size_t rb = ((size_t)h->nc * nxy * real_size(lattice->precision) + 255) / 256 * 256;
+    cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
+    if (ok && marches(h->nc, *lattice) && snapshot_pays(h)) {
+        if (cudaMalloc(&h->snapshots, 2 * rb) == cudaSuccess) h->rho_next = static_cast<char*>(h->snapshots) + rb;
+        else cudaGetLastError();
+    }
+    ok = ok && (h->snapshots || cudaMalloc(&h->snapshots, rb) == cudaSuccess);
+    h->rho_prev = h->snapshots;
     if (!ok) {
         cudaGetLastError();
         release(h);

@@ -75,3 +75,28 @@ def test_a_server_admits_by_what_its_batch_holds(fm):
             with pytest.raises(fm.FmlbmError):
                 fm.fmlbm_server_submit(s, mix, L, rho)
         fm.fmlbm_server_destroy(s)
+
+
+@pytest.mark.parametrize("n,precision,shape", [(2, "fp32", (4096, 2048)), (2, "fp64", (2048, 1024))])
+def test_a_lattice_without_room_for_its_scratch_steps_all_the_same(fm, n, precision, shape):
+    # device memory for all that the lattice needs, not for its second snapshot or scratch planes as well
+    import torch
+    mix = fm.mixture_from_dict(mixture_dict(n, Tr=0.9, kappa_scale=0.3))
+    pinned = torch.from_numpy(smooth_state(n, *shape, seed=4)).pin_memory()   # read in place: no device copy
+    out = []
+    for short in (False, True):
+        filler = None
+        if short:
+            L = fm.make_lattice(*shape, 0.9, precision=precision)
+            scratch = (3 * n + 2) * 8 if precision == "fp64" else n * 4
+            need = fm.fmlbm_lattice_bytes(n, L) - scratch * shape[0] * shape[1] + 10 * (2 << 20)
+            torch.cuda.empty_cache()
+            filler = torch.empty(_free() - need - (16 << 20), dtype=torch.uint8, device="cuda")
+        lat = fm.Lattice(mix, *shape, 0.9, precision=precision)
+        lat.init(pinned.numpy())
+        rows = fm.fmlbm_step_diagnostics(lat.h, 3, n)
+        del filler
+        torch.cuda.empty_cache()
+        out.append(tuple(rows) + lat.distributions())
+        lat.close()
+    assert all(np.array_equal(u, v) for u, v in zip(*out))
