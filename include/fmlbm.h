@@ -556,7 +556,8 @@ typedef struct fmlbm_decomp fmlbm_decomp;
  * slab. */
 fmlbm_status fmlbm_decomp_slab_rows(int32_t ny, int32_t nslabs, int32_t slab, int32_t* y0, int32_t* rows);
 /* Creates nslabs slab lattices of the global lattice (its nx, ny, tau, stencil, precision,
- * velocity force, formulation) for the mixture, each with its own device buffers. */
+ * velocity force, formulation) for the mixture, each with its own device buffers; the scratch
+ * planes of a two-launch step, where there is memory for them, are one slab's and shared. */
 fmlbm_status fmlbm_decomp_create(const fmlbm_mixture* mixture, const fmlbm_lattice* lattice, int32_t nslabs,
                                  void* cuda_stream, fmlbm_decomp** out);
 /* Fluid at rest (as fmlbm_init) from the global densities rho_host [N][ny][nx] (host, copied). */

@@ -70,6 +70,7 @@ struct fmlbm_handle {
     long long wait_polls = kMaxPolls;  // bound of a wait for a tile copy (bulk-copy step forms)
     int check_y0 = 0, check_y1 = 0;    // rows the domain check covers (check_y1 = 0: all)
     void* fields = nullptr;            // split step: scratch planes (null: the step runs fused)
+    bool owns_fields = true;           // false: lent by fmlbm_internal_lend_fields
     long long* done = nullptr;         // per-tile step counters of the multi-step kernel
     CUtensorMap tmap[2][2];          // [buffer][0: float planes, 1: 16-bit planes]
     std::string last_error;
@@ -423,7 +424,7 @@ void release(fmlbm_handle* h) {
     if (h->snapshots) cudaFree(h->snapshots);
     if (h->partial) cudaFree(h->partial);
     if (h->done) cudaFree(h->done);
-    if (h->fields) cudaFree(h->fields);
+    if (h->fields && h->owns_fields) cudaFree(h->fields);
     if (h->diag_dev) cudaFree(h->diag_dev);
     if (h->diag_host) cudaFreeHost(h->diag_host);
     for (int k = 0; k < kDiagSlots; ++k)
@@ -504,6 +505,16 @@ struct ExternalBuffers {
     void* F[2];
 };
 
+ExternalBuffers external_buffers(void* const g[2], float* const g0[2], void* const force[2]) {
+    ExternalBuffers ext;
+    for (int k = 0; k < 2; ++k) {
+        ext.g[k] = g[k];
+        ext.g0[k] = g0 ? g0[k] : nullptr;
+        ext.F[k] = force[k];
+    }
+    return ext;
+}
+
 // cuMemGetAddressRange through the runtime's driver entry point: the base and size of the
 // allocation that contains a device address (null if the driver does not provide it).
 PFN_cuMemGetAddressRange_v3020 address_range_fn() {
@@ -567,8 +578,9 @@ bool disjoint(const void* const* p, const size_t* bytes, int n) {
     return true;
 }
 
+// scratch = false: without the second snapshot and the split step's planes.
 fmlbm_status create_handle(const fmlbm_mixture* mixture, const fmlbm_lattice* lattice, void* cuda_stream,
-                           const ExternalBuffers* ext, fmlbm_handle** out) {
+                           const ExternalBuffers* ext, bool scratch, fmlbm_handle** out) {
     if (!mixture || !lattice || !out) return FMLBM_E_INVALID_ARG;
     *out = nullptr;
     fmlbm_handle* h = new (std::nothrow) fmlbm_handle();
@@ -640,7 +652,7 @@ fmlbm_status create_handle(const fmlbm_mixture* mixture, const fmlbm_lattice* la
     // binary took 372 us instead of 306); without memory for both, one
     const size_t rb = ((size_t)h->nc * nxy * real_size(lattice->precision) + 255) / 256 * 256;
     cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
-    if (ok && marches(h->nc, *lattice) && snapshot_pays(h)) {
+    if (ok && scratch && marches(h->nc, *lattice) && snapshot_pays(h)) {
         if (cudaMalloc(&h->snapshots, 2 * rb) == cudaSuccess) h->rho_next = static_cast<char*>(h->snapshots) + rb;
         else cudaGetLastError();
     }
@@ -658,7 +670,7 @@ fmlbm_status create_handle(const fmlbm_mixture* mixture, const fmlbm_lattice* la
         return FMLBM_E_CUDA;
     }
     // the split step's planes; without them (no memory left) the lattice steps fused
-    const size_t planes = fields_bytes(h->nc, *lattice);
+    const size_t planes = scratch ? fields_bytes(h->nc, *lattice) : 0;
     if (planes > 0 && cudaMalloc(&h->fields, planes) != cudaSuccess) {
         cudaGetLastError();
         h->fields = nullptr;
@@ -694,9 +706,20 @@ bool fmlbm_internal_usable_device_pointer(const void* p, size_t bytes, int devic
     return true;
 }
 
-void fmlbm_internal_set_check_rows(fmlbm_handle* h, int y0, int y1) {
-    h->check_y0 = y0;
-    h->check_y1 = y1;
+fmlbm_status fmlbm_internal_create_slab(const fmlbm_mixture* mixture, const fmlbm_lattice* lattice, void* cuda_stream,
+                                        void* const g[2], float* const g0[2], void* const force[2], int y0, int y1,
+                                        fmlbm_handle** out) {
+    const ExternalBuffers ext = external_buffers(g, g0, force);
+    const fmlbm_status s = create_handle(mixture, lattice, cuda_stream, &ext, false, out);
+    if (s != FMLBM_OK) return s;
+    (*out)->check_y0 = y0;
+    (*out)->check_y1 = y1;
+    return FMLBM_OK;
+}
+size_t fmlbm_internal_fields_bytes(int nc, const fmlbm_lattice& L) { return fields_bytes(nc, L); }
+void fmlbm_internal_lend_fields(fmlbm_handle* h, void* fields) {
+    h->fields = fields;
+    h->owns_fields = false;
 }
 
 bool fmlbm_internal_mixture_constants(const fmlbm_mixture& m, MixConst* mc, std::string* why) {
@@ -741,20 +764,15 @@ fmlbm_status fmlbm_lattice_bytes(int32_t n_components, const fmlbm_lattice* latt
 
 fmlbm_status fmlbm_create(const fmlbm_mixture* mixture, const fmlbm_lattice* lattice, void* cuda_stream,
                           fmlbm_handle** out) {
-    return create_handle(mixture, lattice, cuda_stream, nullptr, out);
+    return create_handle(mixture, lattice, cuda_stream, nullptr, true, out);
 }
 
 fmlbm_status fmlbm_create_with_buffers(const fmlbm_mixture* mixture, const fmlbm_lattice* lattice, void* cuda_stream,
                                        void* const g[2], float* const g0[2], void* const force[2],
                                        fmlbm_handle** out) {
     if (!g || !force) return FMLBM_E_INVALID_ARG;
-    ExternalBuffers ext;
-    for (int k = 0; k < 2; ++k) {
-        ext.g[k] = g[k];
-        ext.g0[k] = g0 ? g0[k] : nullptr;
-        ext.F[k] = force[k];
-    }
-    return create_handle(mixture, lattice, cuda_stream, &ext, out);
+    const ExternalBuffers ext = external_buffers(g, g0, force);
+    return create_handle(mixture, lattice, cuda_stream, &ext, true, out);
 }
 
 fmlbm_status fmlbm_buffer_sizes(int32_t n_components, const fmlbm_lattice* lattice, size_t* g_bytes,

@@ -39,6 +39,7 @@ struct fmlbm_decomp {
     int rows = 0;            // own rows per slab
     cudaStream_t stream = nullptr;
     std::vector<Slab> slab;
+    void* fields = nullptr;  // two-launch step: scratch planes that the slabs take in turn
     int64_t steps = 0;       // steps since init: buffer (steps & 1) holds the state
     size_t esize = 0;        // bytes per element of the g planes
     int gplanes = 0;         // planes of g (9N, or 8N for the deviation forms)
@@ -67,6 +68,7 @@ void release(fmlbm_decomp* d) {
             if (s.F[k]) cudaFree(s.F[k]);
         }
     }
+    if (d->fields) cudaFree(d->fields);
 }
 
 // Rows [src_row, src_row + 3) of every plane of slab `from` into rows [dst_row, dst_row + 3)
@@ -143,8 +145,8 @@ fmlbm_status fmlbm_decomp_create(const fmlbm_mixture* mixture, const fmlbm_latti
             ok = cudaMalloc(&s.g[k], gb) == cudaSuccess && cudaMalloc(&s.F[k], fb) == cudaSuccess;
             if (ok && g0b) ok = cudaMalloc((void**)&s.g0[k], g0b) == cudaSuccess;
         }
-        fmlbm_status st = ok ? fmlbm_create_with_buffers(mixture, &d->local, cuda_stream, s.g, g0b ? s.g0 : nullptr,
-                                                         s.F, &s.h)
+        fmlbm_status st = ok ? fmlbm_internal_create_slab(mixture, &d->local, cuda_stream, s.g, g0b ? s.g0 : nullptr, s.F,
+                                                          kGhost, kGhost + rows, &s.h)
                              : FMLBM_E_OOM;
         if (st != FMLBM_OK) {
             cudaGetLastError();
@@ -152,7 +154,18 @@ fmlbm_status fmlbm_decomp_create(const fmlbm_mixture* mixture, const fmlbm_latti
             delete d;
             return st;
         }
-        fmlbm_internal_set_check_rows(s.h, kGhost, kGhost + rows);
+    }
+    // after all that the slabs need, and once for all of them: they step one after the other on one
+    // stream (with planes of its own for each, FP64 lattices that used to fit were refused).  Without
+    // memory for it they step fused.
+    const size_t planes = fmlbm_internal_fields_bytes(d->nc, d->local);
+    if (planes > 0) {
+        if (cudaMalloc(&d->fields, planes) == cudaSuccess)
+            for (Slab& s : d->slab) fmlbm_internal_lend_fields(s.h, d->fields);
+        else {
+            cudaGetLastError();
+            d->fields = nullptr;
+        }
     }
     *out = d;
     return FMLBM_OK;

@@ -16,6 +16,12 @@ size_t fmlbm_internal_batched_bytes(int nc, const fmlbm_lattice& L);
 // A device (or managed) allocation on `device`, aligned to `align` bytes, with at least
 // `bytes` from p to the end of the allocation that contains it.
 bool fmlbm_internal_usable_device_pointer(const void* p, size_t bytes, int device, size_t align = 16);
-// Restricts the domain check of a handle's steps to rows [y0, y1) (y1 = 0: all rows): a slab
-// of a decomposed lattice checks its own rows, not its ghost rows.
-void fmlbm_internal_set_check_rows(fmlbm_handle* h, int y0, int y1);
+// A slab of a decomposed lattice in the decomposition's buffers: without scratch of its own, and with
+// the domain check of its steps restricted to rows [y0, y1), its own rows without the ghost rows.
+fmlbm_status fmlbm_internal_create_slab(const fmlbm_mixture* mixture, const fmlbm_lattice* lattice, void* cuda_stream,
+                                        void* const g[2], float* const g0[2], void* const force[2], int y0, int y1,
+                                        fmlbm_handle** out);
+// Bytes of the two-launch step's scratch planes for a lattice (0: it does not take that step), and
+// planes for a handle that outlive it.  Handles that step one after the other on one stream may share them.
+size_t fmlbm_internal_fields_bytes(int nc, const fmlbm_lattice& L);
+void fmlbm_internal_lend_fields(fmlbm_handle* h, void* fields);

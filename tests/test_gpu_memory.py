@@ -100,3 +100,18 @@ def test_a_lattice_without_room_for_its_scratch_steps_all_the_same(fm, n, precis
         out.append(tuple(rows) + lat.distributions())
         lat.close()
     assert all(np.array_equal(u, v) for u, v in zip(*out))
+
+
+@pytest.mark.parametrize("n,precision,shape", [(2, "fp64", (2048, 2048)), (2, "fp32", (4096, 4096))])
+def test_the_slabs_of_a_lattice_share_their_scratch(fm, n, precision, shape):
+    # four slabs: what they need, the scratch planes of one (FP64), and no second snapshot of any
+    nx, ny = shape
+    mix = fm.mixture_from_dict(mixture_dict(n, Tr=0.9, kappa_scale=0.3))
+    local = fm.make_lattice(nx, ny // 4 + 6, 0.9, precision=precision)
+    scratch = ((3 * n + 2) * 8 if precision == "fp64" else n * 4) * nx * (ny // 4 + 6)
+    need = 4 * (fm.fmlbm_lattice_bytes(n, local) - scratch) + (scratch if precision == "fp64" else 0)
+    _lattice(fm, n, 64, 64, precision).close()
+    before = _free()
+    d = fm.Decomposition(mix, nx, ny, 0.9, 4, precision=precision)
+    assert before - _free() <= need + 4 * 10 * (2 << 20)   # ten allocations a slab, rounded up to 2 MiB
+    d.close()
